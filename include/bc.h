@@ -425,12 +425,12 @@ bc_status bc_apply_host(bc_plan* plan, void* const* host_ptrs,
 
 /*
  * Boundary conditions fused with the stencil that reads them (Sec. IV-C:
- * the boundary rows only feed the next stencil).  One launch computes, for
+ * the boundary rows only feed the next stencil).  One call computes, for
  * every data value x of every slot,
  *     out[x] = sum_p coeffs[p] * f(x + offsets[p])
  * where f is the field as bc_apply leaves it: data values as stored,
  * covered ghost values evaluated from their row of A and b where the
- * stencil reads them, uncovered ghost values as stored.  The same launch
+ * stencil reads them, uncovered ghost values as stored.  The same call
  * writes every covered ghost value of the fields (bit for bit as bc_apply
  * does for copies and zero rows), so afterwards the fields are those of a
  * bc_apply.  With a plan from bc_plan_create_pruned for the same stencil,
@@ -441,8 +441,10 @@ bc_status bc_apply_host(bc_plan* plan, void* const* host_ptrs,
  * not touched; out must not overlap the fields).  offsets: npoints triples
  * (di, dj, dk), coeffs: npoints FP64 weights (rounded to the plan's dtype),
  * both host memory read during the call (they travel as launch
- * parameters: no allocation, graph-capturable).  Each point's sum runs in
- * the order of the points.  Needs bc_plan_opts.stencil_fusion = 1 at
+ * parameters: no allocation, graph-capturable).  Each value's sum runs in
+ * the order of the points, except that a full 3 x 3 x 3 box with one weight
+ * off the centre (and a centre weight at least as large) is summed axis by
+ * axis.  Needs bc_plan_opts.stencil_fusion = 1 at
  * creation (else BC_ERR_UNSUPPORTED, as for plans with Sync rows);
  * BC_ERR_INVALID_ARG for npoints outside 1..125 or a non-finite weight;
  * BC_ERR_HALO_TOO_WIDE when an offset reaches past a block's ghost width,

@@ -17,7 +17,9 @@ OUT_DIR = os.path.join(HERE, "_lib")
 SOURCES = ["plan.cpp", "prune.cpp", "quadrature.cpp", "kernels.cu", "geometry.cu", "sync.cu",
            "fused.cu", "pack.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
-FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC",
+# kernels.cu holds most of the device code: its optimisation is split over
+# the host's cores
+FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "--split-compile", "0",
          "-I", os.path.join(ROOT, "include")]
 
 

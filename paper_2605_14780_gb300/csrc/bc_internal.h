@@ -206,6 +206,10 @@ struct FuseSlot {
   int32_t nd, nf;     // data cells and ghost-frame cells of one level
   int32_t nt[3];      // tiles along each axis (tz cells deep along axis 2)
   int32_t tz;         // kTileZ, or 1 for 2-D blocks
+  // box path (k_fused_box): the slot's first CTA, tiles along the axes and
+  // planes of one tile
+  int64_t bcta0;
+  int32_t bnt[3], bz;
   FastDiv dL, dnd, dnf, dn0, dn01;  // division by L, nd, nf, n[0], n[0] * n[1]
 };
 struct FuseCtx {
@@ -222,11 +226,24 @@ struct FuseCtx {
 struct FuseStencil {
   int32_t n;
   int32_t r[3];       // halo of the stencil along each axis (<= 2)
+  // 1: a full 3 x 3 x 3 box with one weight `a` off the centre and a centre
+  // weight at least as large; `d` = centre weight - a
+  int32_t box;
+  double a, d;
   int8_t o[kFuseMaxPoints][3];
   double c[kFuseMaxPoints];
 };
 cudaError_t launch_fused(int dtype, const FuseCtx& F, const FuseStencil& st, void* const* slots,
                          void* const* outs, int64_t nctas, cudaStream_t s);
+// Box path: CTAs of kBoxThreads, one per tile of kBoxX x kBoxY cells and
+// FuseSlot::bz planes and level; reads the ghosts from memory (filled by an
+// earlier launch on the stream).
+constexpr int kBoxThreads = 64;
+constexpr int kBoxTy = 4;  // outputs of a thread along y (2 along x)
+constexpr int kBoxX = 32, kBoxY = kBoxThreads / 16 * kBoxTy;
+cudaError_t launch_fused_box(int dtype, const FuseCtx& F, const FuseStencil& st,
+                             void* const* slots, void* const* outs, int64_t nctas,
+                             cudaStream_t s);
 
 // Box packing (pack.cu): one descriptor per box; CTAs are cut per box.
 constexpr int kPackThreads = 256;

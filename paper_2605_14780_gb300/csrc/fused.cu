@@ -10,7 +10,9 @@
 // use, uncovered ghost values as stored.  The same launch also writes every
 // covered ghost value (f's ghosts), so the fields end as after bc_apply.
 // Stencil threads never read covered ghost memory (they evaluate the row),
-// so the ghost writes and the stencil reads do not race.
+// so the ghost writes and the stencil reads do not race.  27-point box
+// stencils with one weight off the centre take two launches instead: the
+// plan's ghost fill, then k_fused_box (below) over the filled fields.
 //
 // Rows are the plan's level-0 rows of A in CSR form; each slot has a table
 // that maps every cell of its ghost frame (the full region minus the data
@@ -228,6 +230,210 @@ __global__ void __launch_bounds__(kFuseThreads)
   xb[cell_off(S, i, j, k) + (int64_t)l * S.ls] = copy ? bits : to_bits_f(val);
 }
 
+// Box stencils (FuseStencil::box): a x (sum over the 3 x 3 x 3 box) +
+// (c0 - a) x centre.  In FP64 the general kernel is bound by the FP64 pipe
+// (27 multiply-adds a value at 1.15 TFLOP/s; GB300 issues one FP64 warp
+// instruction per 16 cycles and SM), so this one counts FP64 instructions:
+// the box sum is taken axis by axis and neighbouring outputs share their
+// pair sums (x: s = x0 + x1, rows x(-1) + s and s + x2; y and z alike),
+// 1.5 adds per value and axis, 6.25 FP64 instructions per value at |a| = 1
+// with 2 x 4 values a thread (2.25 for the row sums with their two halo
+// rows, 1.5 + 1.5, 1 for the centre), 7.25 otherwise.  2 x 2 values a thread
+// (7 instructions, twice the warps) took 8 % longer on the blocks below,
+// 2 x 8 40 %, a ring of six planes with the next pair in flight 4 %.
+//
+// The ghosts are filled by the plan's own launch first and read from memory
+// (evaluating them while staging, as the general kernel does, put chains of
+// dependent loads and divergence into every tile at a face: 1107 us).  A CTA
+// of 2 warps takes 32 x 16 cells (a warp 32 x 8) and walks bz planes in
+// pairs; a ring of four planes with their halo sits in shared memory (20 KB
+// in FP64, eight CTAs an SM: while one waits for its planes the others keep
+// the pipe busy; 4 warps a CTA: 2 % longer, 1 warp: 1 %).  The sums associate
+// differently from the general kernel's (against sums in higher precision
+// they are the closer ones: 1.4e-16 to 2.2e-16 of the result's norm for the
+// operator below); a value that is not finite is summed again in the general
+// order from the ring, so infinities, NaNs and overflow come out as there.
+//
+// 27-point operator (26, -1) on 16 blocks of 128^3 FP64, fill included:
+// 1579 -> 474 us, the FP64 pipe 75 % busy.
+template <typename T>
+__device__ __forceinline__ void cp_async_cell(T* smem, const T* gmem) {
+  const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
+  if constexpr (sizeof(T) == 4)
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(sa), "l"(gmem) : "memory");
+  else
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(sa), "l"(gmem) : "memory");
+}
+
+constexpr int kBoxPitch = kBoxX + 2, kBoxPlane = kBoxPitch * (kBoxY + 2);
+constexpr int kBoxCtas = 512 / kBoxThreads;  // 16 warps an SM
+
+template <typename T> struct Pair2;
+template <> struct Pair2<float> { using type = float2; };
+template <> struct Pair2<double> { using type = double2; };
+
+// 3 x 3 sums of one staged plane for a thread's 2 x 4 cells; `c`: the
+// staged value one row above and one cell before the thread's first
+template <typename T>
+__device__ __forceinline__ void plane_sums(const T* c, T (&P)[2 * kBoxTy]) {
+  using V = typename Pair2<T>::type;
+  T r[kBoxTy + 2][2];
+#pragma unroll
+  for (int j = 0; j < kBoxTy + 2; ++j) {
+    const V a = *reinterpret_cast<const V*>(c + j * kBoxPitch);
+    const V b = *reinterpret_cast<const V*>(c + j * kBoxPitch + 2);
+    const T s = a.y + b.x;
+    r[j][0] = a.x + s;
+    r[j][1] = s + b.y;
+  }
+#pragma unroll
+  for (int x = 0; x < 2; ++x)
+#pragma unroll
+    for (int j = 0; j < kBoxTy; j += 2) {
+      const T s = r[j + 1][x] + r[j + 2][x];
+      P[2 * j + x] = r[j][x] + s;
+      P[2 * (j + 1) + x] = s + r[j + 3][x];
+    }
+}
+
+// by the exponent bits: a floating compare would take the FP64 pipe
+__device__ __forceinline__ bool finite_value(float v) {
+  return (__float_as_uint(v) & 0x7f800000u) != 0x7f800000u;
+}
+__device__ __forceinline__ bool finite_value(double v) {
+  return ((unsigned)__double2hiint(v) & 0x7ff00000u) != 0x7ff00000u;
+}
+
+// v, or -v where `flip` holds the sign bit (no FP64 instruction either)
+__device__ __forceinline__ float flip_sign(float v, unsigned flip) {
+  return __uint_as_float(__float_as_uint(v) ^ flip);
+}
+__device__ __forceinline__ double flip_sign(double v, unsigned flip) {
+  return __hiloint2double((int)((unsigned)__double2hiint(v) ^ flip), __double2loint(v));
+}
+
+// UNIT: |a| = 1, a x S is S or -S
+template <typename T, bool UNIT>
+__global__ void __launch_bounds__(kBoxThreads, kBoxCtas)
+    k_fused_box(FuseCtx F, FuseStencil st, void* const* slots, void* const* outs) {
+  __shared__ FuseSlot S;
+  __shared__ int si;
+  __shared__ __align__(16) T ring[4][kBoxPlane];
+  const int tid = threadIdx.x;
+  if (tid == 0) {
+    int lo = 0, hi = F.nslots - 1;  // the last slot whose first CTA is <= blockIdx.x
+    while (lo < hi) {
+      const int mid = (lo + hi + 1) >> 1;
+      if (F.slot[mid].bcta0 <= (int64_t)blockIdx.x) lo = mid;
+      else hi = mid - 1;
+    }
+    si = lo;
+    S = F.slot[lo];
+  }
+  __syncthreads();
+  int t = blockIdx.x - (int)S.bcta0;
+  const int tx = t % S.bnt[0];
+  t /= S.bnt[0];
+  const int ty = t % S.bnt[1];
+  t /= S.bnt[1];
+  const int tz = t % S.bnt[2];
+  const int l = t / S.bnt[2];
+  const int i0 = tx * kBoxX, j0 = ty * kBoxY, k0 = tz * S.bz;
+  const int k1 = min(k0 + S.bz, S.n[2]);
+  const int warp = tid >> 5, lane = tid & 31;
+  const int64_t s0 = S.s[0], s1 = S.s[1], s2 = S.s[2];
+  const int64_t org = cell_off(S, i0, j0, k0) + (int64_t)l * S.ls;
+  const T* x = static_cast<const T*>(slots[si]) + org;
+
+  // planes k and k + 1 with their halo into the ring (plane k in slot k & 3),
+  // a warp a row; cells past the full region only border outputs past the
+  // data region and are zero
+  const int iend = S.n[0] + S.h[0] - i0, jend = S.n[1] + S.h[1] - j0;
+  auto stage = [&](int k) {
+    for (int r = warp; r < 2 * (kBoxY + 2); r += kBoxThreads / 32) {
+      const int z = r >= kBoxY + 2, j = r - z * (kBoxY + 2) - 1, kk = k + z;
+      T* dst = ring[kk & 3] + (j + 1) * kBoxPitch;
+      const bool row = j < jend && kk < S.n[2] + S.h[2];
+      const T* src = x + ((int64_t)(kk - k0) * s2 + (int64_t)j * s1);
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        const int li = lane + 32 * u;
+        if (li >= kBoxPitch) break;
+        if (row && li - 1 < iend)
+          cp_async_cell<T>(dst + li, src + (int64_t)(li - 1) * s0);
+        else
+          dst[li] = T(0);
+      }
+    }
+    asm volatile("cp.async.wait_all;\n" ::: "memory");
+  };
+
+  // this thread's cells: 2 along x from cx, kBoxTy along y from cy
+  const int cx = 2 * (lane & 15), cy = warp * 2 * kBoxTy + (lane >> 4) * kBoxTy;
+  const int at = cy * kBoxPitch + cx;  // staged value at (-1, -1) of the first cell
+  // a warp whose rows all lie past the block has nothing to sum
+  const bool work = j0 + warp * 2 * kBoxTy < S.n[1];
+  const int nx = S.n[0] - i0 - cx, ny = S.n[1] - j0 - cy;  // this thread's cells in the block
+  T* out = static_cast<T*>(outs[si]) + (org + cx * s0 + cy * s1);
+  const T a = (T)st.a, d = (T)st.d;
+  const unsigned flip = st.a < 0 ? 0x80000000u : 0u;
+
+  // the outputs of plane k from the box sums b
+  auto put = [&](int k, const T (&b)[2 * kBoxTy]) {
+    const T* c = ring[k & 3] + at + kBoxPitch + 1;
+    T* o = out + (int64_t)(k - k0) * s2;
+#pragma unroll
+    for (int j = 0; j < kBoxTy; ++j)
+#pragma unroll
+      for (int xx = 0; xx < 2; ++xx) {
+        const T x0 = c[j * kBoxPitch + xx], s = b[2 * j + xx];
+        T v = UNIT ? fma(d, x0, flip_sign(s, flip)) : fma(a, s, d * x0);
+        if (!finite_value(v)) {
+          v = T(0);
+          for (int p = 0; p < st.n; ++p)
+            v = fma((T)st.c[p],
+                    ring[(k + st.o[p][2]) & 3]
+                    [at + (j + 1 + st.o[p][1]) * kBoxPitch + xx + 1 + st.o[p][0]],
+                    v);
+        }
+        if (xx < nx && j < ny) o[j * s1 + xx * s0] = v;
+      }
+  };
+
+  T p0[2 * kBoxTy], p1[2 * kBoxTy];  // plane sums of k - 1 and k
+  stage(k0 - 1);
+  __syncthreads();
+  if (work) {
+    plane_sums<T>(ring[(k0 - 1) & 3] + at, p0);
+    plane_sums<T>(ring[k0 & 3] + at, p1);
+  }
+  for (int k = k0; k < k1; k += 2) {
+    stage(k + 1);
+    __syncthreads();
+    if (work) {
+      T p2[2 * kBoxTy], b[2 * kBoxTy];
+      plane_sums<T>(ring[(k + 1) & 3] + at, p2);
+#pragma unroll
+      for (int q = 0; q < 2 * kBoxTy; ++q) {
+        p1[q] += p2[q];         // planes k and k + 1, shared by both outputs
+        b[q] = p0[q] + p1[q];
+        p0[q] = p2[q];
+      }
+      put(k, b);
+      if (k + 1 < k1) {
+        plane_sums<T>(ring[(k + 2) & 3] + at, p2);
+#pragma unroll
+        for (int q = 0; q < 2 * kBoxTy; ++q) {
+          b[q] = p1[q] + p2[q];
+          p1[q] = p2[q];
+        }
+        put(k + 1, b);
+      }
+    }
+    __syncthreads();  // planes k - 1 and k are free for k + 3 and k + 4
+  }
+}
+
 }  // namespace
 
 cudaError_t launch_fused(int dtype, const FuseCtx& F, const FuseStencil& st, void* const* slots,
@@ -237,6 +443,17 @@ cudaError_t launch_fused(int dtype, const FuseCtx& F, const FuseStencil& st, voi
     k_fused<double><<<(unsigned)nctas, kFuseThreads, 0, s>>>(F, st, slots, outs);
   else
     k_fused<float><<<(unsigned)nctas, kFuseThreads, 0, s>>>(F, st, slots, outs);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_fused_box(int dtype, const FuseCtx& F, const FuseStencil& st,
+                             void* const* slots, void* const* outs, int64_t nctas,
+                             cudaStream_t s) {
+  if (nctas <= 0) return cudaSuccess;
+  const bool unit = st.a == 1.0 || st.a == -1.0;
+  auto* kernel = dtype == 1 ? (unit ? k_fused_box<double, true> : k_fused_box<double, false>)
+                            : (unit ? k_fused_box<float, true> : k_fused_box<float, false>);
+  kernel<<<(unsigned)nctas, kBoxThreads, 0, s>>>(F, st, slots, outs);
   return cudaGetLastError();
 }
 

@@ -203,7 +203,7 @@ struct bc_plan {
   // device
   DevBuf tables, work, fuse;
   FuseCtx fuse_ctx{};
-  int64_t fuse_ctas = 0;
+  int64_t fuse_ctas = 0, fuse_box_ctas = 0;
   Ctx ctx{};
   Item* d_items = nullptr;
   Item* d_fam[kFamilies] = {nullptr, nullptr, nullptr, nullptr};
@@ -2038,6 +2038,34 @@ bc_status build_fusion(bc_plan* P) {
     cta += f.tiles + ((F - D) * B.nlevels + kFuseThreads - 1) / kFuseThreads;
   }
   P->fuse_ctas = cta;
+  // Box path: planes per tile.  A tile's cost is its planes plus the two it
+  // only sums (and about eight planes' worth of start-up), the grid's the
+  // tiles of the fullest SM: 16 blocks of 128^3 take 32 planes (2048 tiles).
+  {
+    double best = 0;
+    int bz = 4;
+    for (int z : {4, 6, 8, 12, 16, 24, 32, 48, 64}) {
+      int64_t tiles = 0;
+      for (const FuseSlot& f : slots)
+        tiles += (int64_t)((f.n[0] + kBoxX - 1) / kBoxX) * ((f.n[1] + kBoxY - 1) / kBoxY) *
+                 ((f.n[2] + z - 1) / z) * f.L;
+      const double cost = (double)((tiles + P->num_sms - 1) / P->num_sms) * (z + 1.2 + 8.0);
+      if (z == 4 || cost < best) {
+        best = cost;
+        bz = z;
+      }
+    }
+    int64_t b0 = 0;
+    for (FuseSlot& f : slots) {
+      f.bz = bz;
+      f.bnt[0] = (f.n[0] + kBoxX - 1) / kBoxX;
+      f.bnt[1] = (f.n[1] + kBoxY - 1) / kBoxY;
+      f.bnt[2] = (f.n[2] + bz - 1) / bz;
+      f.bcta0 = b0;
+      b0 += (int64_t)f.bnt[0] * f.bnt[1] * f.bnt[2] * f.L;
+    }
+    P->fuse_box_ctas = b0;
+  }
   // frame index of a ghost cell (the device's frame_index)
   auto frame_index = [](const FuseSlot& f, int i, int j, int k) -> int64_t {
     const int64_t F0 = f.n[0] + 2 * f.h[0], F1 = f.n[1] + 2 * f.h[1];
@@ -2107,6 +2135,41 @@ bc_status build_fusion(bc_plan* P) {
   F.rhs = b + o_b;
   F.slot_ls = P->ctx.slot_ls;
   return BC_OK;
+}
+
+// Whether the stencil is a box (FuseStencil::box): the 27 points of
+// [-1, 1]^3 once each, one weight a off the centre and a centre weight c0
+// with |c0| >= |a| (the box form adds a x0 to the sum and takes it out again
+// with c0 - a, so its rounding stays within |c0 x0|'s share only then),
+// weights as the kernels hold them (the plan's dtype).
+void box_stencil(int dtype, FuseStencil& st) {
+  if (st.n != 27) return;
+  auto held = [&](double v) { return dtype == BC_F64 ? v : (double)(float)v; };
+  unsigned seen = 0;
+  double a = 0, c0 = 0;
+  bool first = true;
+  for (int p = 0; p < 27; ++p) {
+    const int i = st.o[p][0] + 1, j = st.o[p][1] + 1, k = st.o[p][2] + 1;
+    if (i < 0 || i > 2 || j < 0 || j > 2 || k < 0 || k > 2) return;
+    const int at = (k * 3 + j) * 3 + i;
+    seen |= 1u << at;
+    const double c = held(st.c[p]);
+    if (at == 13) {
+      c0 = c;
+    } else if (first) {
+      a = c;
+      first = false;
+    } else if (c != a) {
+      return;
+    }
+  }
+  const double d = held(c0 - a);
+  if (seen != (1u << 27) - 1 || a == 0 || std::fabs(c0) < std::fabs(a) || !std::isfinite(a) ||
+      !std::isfinite(d))
+    return;
+  st.box = 1;
+  st.a = a;
+  st.d = d;
 }
 
 // FNV-1a over the bytes that decide what the autotuner measures: dtype,
@@ -3048,8 +3111,26 @@ bc_status bc_apply_stencil(bc_plan* plan, void* const* slot_ptrs, void* const* o
     }
     st.c[p] = coeffs[p];
   }
-  cudaError_t e = launch_fused(plan->dtype, plan->fuse_ctx, st, slot_ptrs, out_ptrs,
-                               plan->fuse_ctas, static_cast<cudaStream_t>(stream));
+  box_stencil(plan->dtype, st);
+  cudaStream_t s = static_cast<cudaStream_t>(stream);
+  cudaError_t e;
+  if (st.box) {
+    // the ghost fill, then the box sums that read it; the families one
+    // after another on the caller's stream, without the plan's own streams
+    // and events, so that calls on several streams and threads stay apart
+    Ctx c = plan->ctx;
+    c.slots = slot_ptrs;
+    c.vec_runs = plan->opts.scalar_runs ? 0 : 1;
+    e = cudaSuccess;
+    for (int f = 0; f < kFamilies && e == cudaSuccess; ++f)
+      e = launch_family(plan->dtype, f, c, plan->d_fam[f], (int)plan->fam_items[f].size(),
+                        plan->opts.threads, 0, plan->staged[f], s);
+    if (e == cudaSuccess)
+      e = launch_fused_box(plan->dtype, plan->fuse_ctx, st, slot_ptrs, out_ptrs,
+                           plan->fuse_box_ctas, s);
+  } else {
+    e = launch_fused(plan->dtype, plan->fuse_ctx, st, slot_ptrs, out_ptrs, plan->fuse_ctas, s);
+  }
   if (e != cudaSuccess) return cuda_fail(e, "stencil launch");
   return BC_OK;
 }
