@@ -245,19 +245,27 @@ cudaError_t launch_fused_box(int dtype, const FuseCtx& F, const FuseStencil& st,
                              void* const* slots, void* const* outs, int64_t nctas,
                              cudaStream_t s);
 
-// Box packing (pack.cu): one descriptor per box; CTAs are cut per box.
+// Box packing (pack.cu): one descriptor per box; CTAs take tiles of at most
+// nc cells x nl levels of one component, {box, component, first cell, first
+// level} each.
 constexpr int kPackThreads = 256;
+constexpr int kPackVals = 2048;   // nc * nl, at most
+constexpr int kPackCells = 512;   // nc, at most
+constexpr int kPackLevels = 64;   // nl where the levels are contiguous, at most
 struct PackBox {
   int32_t slot0;          // slot of component 0 of the box's block
   int32_t lo[3], e[3];    // first cell (data coordinates) and extents
   int32_t L, ncomp;
+  int32_t cells;          // e[0] * e[1] * e[2]
+  int32_t nc, nl;         // cells and levels of a tile
+  int32_t lfast;          // 1: levels contiguous in the field
   int64_t s[3], ls;       // element strides of the block (ls: 0 for one level)
   int64_t dst;            // first buffer element of the box
-  int64_t count;          // values: ncomp * L * e[0] * e[1] * e[2]
-  int64_t cta0;           // the box's first CTA
-  FastDiv d0, d1, d2, dL; // division by e[0], e[1], e[2], L
+  FastDiv d0, d1, dnc, dnl;  // division by e[0], e[1], nc, nl
 };
-cudaError_t launch_pack(int esize, const PackBox* boxes, int nboxes, int64_t nctas,
+static_assert(sizeof(PackBox) % 4 == 0 && sizeof(PackBox) / 4 <= kPackThreads,
+              "a PackBox is loaded as one word per thread");
+cudaError_t launch_pack(int esize, const PackBox* boxes, const int4* tiles, int64_t ntiles,
                         void* const* slots, void* buf, cudaStream_t s);
 
 // Sets the message bc_last_error() returns on this thread (plan.cpp).

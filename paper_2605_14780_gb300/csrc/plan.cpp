@@ -3139,8 +3139,8 @@ bc_status bc_apply_stencil(bc_plan* plan, void* const* slot_ptrs, void* const* o
 
 struct bc_pack {
   int esize = 4;
-  int64_t size = 0, nctas = 0;
-  int nboxes = 0;
+  int64_t size = 0, ntiles = 0;
+  const int4* tiles = nullptr;  // behind the box descriptors
   DevBuf boxes;
 };
 
@@ -3160,7 +3160,8 @@ bc_status bc_pack_create(const bc_grid* grid, const bc_box* boxes, int32_t nboxe
     ns += grid->blocks[b].ncomp;
   }
   std::vector<PackBox> desc(nboxes);
-  int64_t pos = 0, cta = 0;
+  std::vector<int4> tiles;
+  int64_t pos = 0;
   for (int t = 0; t < nboxes; ++t) {
     const bc_box& x = boxes[t];
     if (x.block < 0 || x.block >= grid->nblocks)
@@ -3182,35 +3183,54 @@ bc_status bc_pack_create(const bc_grid* grid, const bc_box* boxes, int32_t nboxe
     d.L = B.nlevels;
     d.ncomp = B.ncomp;
     d.ls = B.nlevels > 1 ? B.level_stride : 0;
-    d.count = cells * B.nlevels * B.ncomp;
-    if (d.count >= INT32_MAX) return fail(BC_ERR_UNSUPPORTED, "box %d holds 2^31 values or more", t);
+    const int64_t count = cells * B.nlevels * B.ncomp;
+    if (count >= INT32_MAX) return fail(BC_ERR_UNSUPPORTED, "box %d holds 2^31 values or more", t);
     // offsets relative to the slot pointer, which addresses cell (-h, -h, -h)
     for (int a = 0; a < 3; ++a) d.lo[a] += B.h[a];
     d.dst = pos;
-    d.cta0 = cta;
+    d.cells = (int32_t)cells;
+    d.lfast = d.ls == 1;
+    // Tiles: with contiguous levels all of them (in equal parts of at most
+    // kPackLevels), as many cells as fill kPackVals; otherwise the cells
+    // (the runs of both sides) first.
+    if (d.lfast) {
+      const int parts = std::max(1, (d.L + kPackLevels - 1) / kPackLevels);
+      d.nl = std::max(1, (d.L + parts - 1) / parts);
+      d.nc = (int32_t)std::min<int64_t>(std::min(kPackCells, kPackVals / d.nl), cells);
+    } else {
+      d.nc = (int32_t)std::min<int64_t>(kPackCells, cells);
+      d.nl = std::max(1, std::min(kPackVals / d.nc, d.L));
+    }
     d.d0 = make_div((uint32_t)d.e[0]);
     d.d1 = make_div((uint32_t)d.e[1]);
-    d.d2 = make_div((uint32_t)d.e[2]);
-    d.dL = make_div((uint32_t)d.L);
-    pos += d.count;
-    cta += (d.count + kPackThreads - 1) / kPackThreads;
+    d.dnc = make_div((uint32_t)d.nc);
+    d.dnl = make_div((uint32_t)d.nl);
+    pos += count;
+    for (int c = 0; c < d.ncomp; ++c)
+      for (int l0 = 0; l0 < d.L; l0 += d.nl)
+        for (int64_t m0 = 0; m0 < cells; m0 += d.nc) tiles.push_back(make_int4(t, c, (int)m0, l0));
   }
   std::unique_ptr<bc_pack> P(new (std::nothrow) bc_pack);
   if (!P) return fail(BC_ERR_NOMEM, "host allocation");
   P->esize = grid->dtype == BC_F64 ? 8 : 4;
   P->size = pos;
-  P->nctas = cta;
-  P->nboxes = nboxes;
+  P->ntiles = (int64_t)tiles.size();
   if (nboxes > 0) {
     arm_fault_injection();
-    cudaError_t e = dev_malloc(&P->boxes.base, desc.size() * sizeof(PackBox));
+    Layout L;
+    const size_t o_b = L.take(desc.size() * sizeof(PackBox)), o_t = L.take(tiles.size() * sizeof(int4));
+    std::vector<char> host(L.off, 0);
+    put_raw(host, o_b, desc);
+    put_raw(host, o_t, tiles);
+    cudaError_t e = dev_malloc(&P->boxes.base, host.size());
     if (e != cudaSuccess) {
       P->boxes.base = nullptr;
       return cuda_fail(e, "pack descriptors");
     }
-    if ((e = cudaMemcpy(P->boxes.base, desc.data(), desc.size() * sizeof(PackBox),
-                        cudaMemcpyHostToDevice)) != cudaSuccess)
+    if ((e = cudaMemcpy(P->boxes.base, host.data(), host.size(), cudaMemcpyHostToDevice)) !=
+        cudaSuccess)
       return cuda_fail(e, "pack descriptors upload");
+    P->tiles = reinterpret_cast<const int4*>(static_cast<char*>(P->boxes.base) + o_t);
   }
   *out = P.release();
   return BC_OK;
@@ -3220,10 +3240,10 @@ int64_t bc_pack_size(const bc_pack* pack) { return pack ? pack->size : 0; }
 
 bc_status bc_pack_run(bc_pack* pack, void* const* slot_ptrs, void* buffer, void* stream) {
   if (!pack) return fail(BC_ERR_INVALID_ARG, "pack is NULL");
-  if (pack->nboxes == 0) return BC_OK;
+  if (pack->ntiles == 0) return BC_OK;
   if (!slot_ptrs || !buffer) return fail(BC_ERR_INVALID_ARG, "slot_ptrs or buffer is NULL");
   cudaError_t e = launch_pack(pack->esize, static_cast<const PackBox*>(pack->boxes.base),
-                              pack->nboxes, pack->nctas, slot_ptrs, buffer,
+                              pack->tiles, pack->ntiles, slot_ptrs, buffer,
                               static_cast<cudaStream_t>(stream));
   if (e != cudaSuccess) return cuda_fail(e, "pack launch");
   return BC_OK;
