@@ -115,6 +115,48 @@ __device__ void structured_flat_t(const Item& it, const Ptrs& P, const Ctx& c, i
   }
 }
 
+// Cells times chunks of up to kChunk levels (mode >= 2, levels far apart in
+// memory): a lane looks its cell up once and moves the chunk's values from
+// there, all in flight, so a value costs a load and a store; one value per
+// unit took two look-ups and a division for each.  The strips across axis 0
+// this serves are bound by DRAM: two or three values of a 64-byte granule,
+// read and written back (2.9-3.5 TB/s of such granules is all that reached
+// DRAM with any order, length or address arithmetic of the units tried:
+// chunks of 32 levels and offsets worked out from the box's strides were 4-12
+// % slower).  Halo copies of 64 blocks of 129^2 x 96 planes 62 -> 54 us,
+// the zero pass of the 6 x 768^2 adjoint 31 -> 27 us.
+template <typename T>
+__device__ void structured_chunk(const Item& it, const Ptrs& P, const Ctx& c, int lane) {
+  using B = typename BitsOf<T>::type;
+  constexpr int U = kChunk;
+  const int end = it.u0 + it.nunits;
+  const int dls = it.dst_ls, sls = it.src_ls, chn = it.mode, kind = it.kind;
+  B* dbase = static_cast<B*>(P.d);
+  const B* sbase = static_cast<const B*>(P.s);
+  for (int u = it.u0 + lane; u < end; u += 32) {
+    int q, ch;
+    unit_of(u, it, q, ch);
+    const int l0 = ch * chn;
+    const int nl = min(chn, (int)it.lev.d - l0);
+    B* d = dbase + (dst_cell(it, c, q) + l0 * dls);
+    B v[U];
+    if (kind == IK_MAP) {
+      const B* s = sbase + (__ldg(c.ctab_s + it.ctab + q) + l0 * sls);
+#pragma unroll
+      for (int l = 0; l < U; ++l)
+        if (l < nl) v[l] = ldg(s + (int64_t)l * sls);
+    } else {
+      const B k =
+          kind == IK_CONST ? ldg(static_cast<const B*>(c.const_val) + it.table + q) : B(0);
+#pragma unroll
+      for (int l = 0; l < U; ++l) v[l] = k;
+    }
+#pragma unroll
+    for (int l = 0; l < U; ++l)
+      if (l < nl) d[(int64_t)l * dls] = v[l];
+  }
+}
+
 // Adjoint of unit copies over runs: x_bar[dst + t] += y_bar[src + t], the
 // data values of P.d and the ghost values of P.s, with the lane layout of
 // the copy runs below.  Runs in the transpose-gather kernel (its register
@@ -377,6 +419,8 @@ __device__ __forceinline__ void structured_flat(const Item& it, const Ptrs& P, c
     structured_runs<T>(it, P, c, lane);
   else if (it.mode == MODE_FLAT_LEVEL)
     structured_flat_t<T, true>(it, P, c, lane);
+  else if (it.mode >= 2)
+    structured_chunk<T>(it, P, c, lane);
   else
     structured_flat_t<T, false>(it, P, c, lane);
 }

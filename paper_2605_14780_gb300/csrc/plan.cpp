@@ -1263,15 +1263,22 @@ void build_items(bc_plan* P) {
   const int64_t want_items = (int64_t)std::max(1, P->num_sms) * 16;
   const int small = (int)std::min<int64_t>(
       1 << 30, std::max<int64_t>(32, (total_values + want_items - 1) / want_items + 31) / 32 * 32);
-  const int per_chunk_item = 32 * upl;
   const int per_flat_item = std::min(32 * kFlatUnroll * std::min(upl, BC_FLAT_UPL_MAX), small);
   // table-driven kinds (interpolation, CSR, transpose): one unit per lane, so
   // a warp's dependent table -> data chains run side by side, not in series
   const int per_table_item = 32;
   const int per_table_flat_item = std::min(32 * 8, small);
   auto structured_emit = [&](std::vector<Item>& out, const Item& it, const bc_block& B, int vol) {
-    const int mode = structured_mode(B, P->opts.unit_order);
-    emit_units(out, it, vol, B.nlevels, mode, mode < 2 ? per_flat_item : per_chunk_item);
+    int mode = structured_mode(B, P->opts.unit_order);
+    if (mode == MODE_FLAT_CELL && B.nlevels > 1) {
+      // levels far apart in memory: cells times equal chunks of at most
+      // kChunk levels, one unit a lane (fewer levels in small plans)
+      const int most = std::max(1, std::min(kChunk, small / 32));
+      const int parts = (B.nlevels + most - 1) / most;
+      mode = (B.nlevels + parts - 1) / parts;
+      if (mode < 2) mode = MODE_FLAT_CELL;
+    }
+    emit_units(out, it, vol, B.nlevels, mode, mode < 2 ? per_flat_item : 32);
   };
   // zero / map sub-matrices: runs when they are long, cached per sub-matrix
   const int per_run_item = std::min(BC_RUN_ITEM * upl, small);
@@ -1387,7 +1394,7 @@ void build_items(bc_plan* P) {
   // per lane
   auto work = [&](const Item& it) -> int64_t {
     if (it.mode == MODE_TILE) return (int64_t)it.nunits * it.nl;
-    if (it.mode != MODE_RUNS) return it.nunits;
+    if (it.mode != MODE_RUNS) return (int64_t)it.nunits * (it.mode >= 2 ? it.mode : 1);
     int64_t n = 0;
     for (int r = it.u0; r < it.u0 + it.nunits; ++r) n += P->runs[r].z;
     return n;
@@ -1412,8 +1419,7 @@ void build_items(bc_plan* P) {
   // times the bytes a value moves: one store, plus the loads of its row)
   {
     auto bytes = [&](const Item& it) -> int64_t {
-      int64_t vals = work(it);
-      if (it.mode >= 2) vals *= it.mode;
+      const int64_t vals = work(it);
       switch (it.kind) {
         case IK_ZERO:
         case IK_CONST: return vals;
