@@ -65,15 +65,22 @@ enum ItemMode : int32_t { MODE_TILE = -2, MODE_RUNS = -1, MODE_FLAT_CELL = 0, MO
 constexpr int32_t kBoxIndex = 0xffff;
 constexpr int32_t kBoxRows = 1 << 16;
 constexpr int32_t kBoxSnap = 1 << 17;
-// shared memory of one warp's staged box: interpolation and transpose
-// tiles 2 KB, CSR tiles 4 KB (measured: the 4 x 4 reconstruction rows of a
-// vector pair then stage 16-row tiles of 6 levels instead of 8-row tiles
-// of 5, 135 -> 87 us on the 6 x 384^2 sphere; the interpolation tiles are
-// 3 % faster with 2 KB)
-constexpr int kStageBytesRows = 2048;
-constexpr int kStageBytesCsr = 4096;
-constexpr int kTileCells = 32;     // cells (rows) of one staged item, at most
-constexpr int kTileLevels = 4;     // levels one lane of a staged CSR or transpose tile sums
+// A staged tile: up to kTileCells cells (rows) whose nodes lie in one box.
+// A level of the box takes a plane of fixed size in a warp's stage, so that
+// the levels a lane sums at once (kTileLevels, of stage_levels staged) are
+// constant offsets from one address: kPlaneInterp elements per component
+// for interpolation tiles, kPlaneCsr / kPlaneAdj elements for all slots of a
+// CSR / transpose tile.
+constexpr int kTileCells = 32;
+constexpr int kTileLevels = 4;
+constexpr int stage_levels(int esize) { return esize == 8 ? kTileLevels : 2 * kTileLevels; }
+constexpr int kPlaneInterp = 64, kPlaneCsr = 256, kPlaneAdj = 128;
+// shared memory of one warp's stage
+constexpr int stage_bytes(bool csr, bool pair_or_adj, int esize) {
+  return stage_levels(esize) * esize *
+         (csr ? kPlaneCsr : (pair_or_adj ? kPlaneAdj : kPlaneInterp));
+}
+static_assert(kPlaneAdj == 2 * kPlaneInterp, "pairs and transpose tiles stage the same bytes");
 
 struct alignas(16) Item {
   int32_t kind;
@@ -89,7 +96,9 @@ struct alignas(16) Item {
   int32_t table;           // CONST / INTERP / CSR: first table row of cell 0
   int32_t comp;            // INTERP source components: u | v << 16
   int32_t dst_ls, src_ls;  // level strides (elements)
-  int32_t src_org;         // CSR: ELL entry of row 0 of this component
+  int32_t src_org;         // CSR: ELL entry of row 0 of this component; staged
+                           // CSR / transpose tiles: the tile's first entry of
+                           // tile_box / tile_w
   // MODE_TILE items: levels [l0, l0 + nl) of the cells [u0, u0 + nunits)
   // (vol divides by nunits), reading a box of bw x bh cells at element
   // offset borg (level 0) of a block that steps bs0 / bs1 elements along
@@ -120,8 +129,12 @@ struct Ctx {
   const void* itp_w;
   const void* itp_m;
   const int32_t* itp_box;   // staged cells: node 0 in the item's box
-  const int32_t* csr_box;   // staged CSR entries: place in a level's stage (slot-major)
-  const int32_t* adj_box;   // staged transpose entries: the same
+  // entries of staged CSR and transpose tiles: place in a level's plane
+  // (selector * box cells + box index) and weight; entry e of row q of a
+  // tile of nq rows at src_org + ((e / 4) * nq + q) * 4 + e % 4, so a warp's
+  // load of four entries a row is one contiguous piece
+  const int32_t* tile_box;
+  const void* tile_w;
   // CSR rows (global row numbering): entry count per row, ELL entries
   // (a row's entries start at item.src_org + q * item.p), per-row constant
   const int32_t* csr_nnz;

@@ -67,8 +67,15 @@ struct Ptrs {
   void* d;
   void* d2;
   const void* s;
-  void* stage;  // this warp's shared-memory staging area (Ctx::stage_warp bytes), or null
+  unsigned stage;  // byte offset of this warp's stage (Ctx::stage_warp bytes)
 };
+
+// the warps' stages (staged tiles), where the launch requests them
+extern __shared__ __align__(16) unsigned char g_stage[];
+
+// An item sits in shared memory, which a store through a field pointer may
+// alias as far as the compiler knows; functions take their own copy, so that
+// its fields stay in registers.
 
 // ---------------------------------------------------------------------------
 // zero / constant / map (matrix-free rows, Sec. III-B)
@@ -541,144 +548,16 @@ __device__ void interp_pair_chunk(const Item& it, const Ptrs& P, const Ctx& c, i
 // neighbour block -- a strip of the edge rows or columns (the transposed
 // strip when the nodes step along the neighbour's strided axis).  The warp
 // copies the box, for the item's levels and components, into its shared
-// memory with cp.async (each source value once, lanes over consecutive
-// cells of a box row), then every lane evaluates its (cell, level) rows
-// from shared memory: the p-point sums, the 2x2 rotation of a vector pair,
-// and the store.  Same sums in the same order as the per-lane path.
-template <typename T>
-__device__ __forceinline__ void cp_async_elem(T* smem, const T* gmem) {
-  const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
-  if constexpr (sizeof(T) == 4)
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(sa), "l"(gmem) : "memory");
-  else
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(sa), "l"(gmem) : "memory");
-}
-
-__device__ __forceinline__ void cp_async_wait_all() {
-  asm volatile("cp.async.wait_all;\n" ::: "memory");
-}
-
-template <typename T>
-__device__ void interp_tile(const Item& it, const Ptrs& P, const Ctx& c, int lane) {
-  using B = typename BitsOf<T>::type;
-  T* sm = static_cast<T*>(P.stage);
-  const bool pair = it.kind == IK_INTERP_PAIR;
-  const int nc = pair ? 2 : 1;
-  const int A = it.bw * it.bh;
-  const int cu = it.comp & 0xffff, cv = it.comp >> 16;
-  const int64_t lev0 = (int64_t)it.l0 * it.src_ls + it.borg;
-  const T* xu = static_cast<const T*>(c.slots[it.bsrc + cu]) + lev0;
-  const T* xv = pair ? static_cast<const T*>(c.slots[it.bsrc + cv]) + lev0 : xu;
-  // stage: [level][component][box row][box column]
-  for (int g = 0; g < it.nl * nc; ++g) {
-    const int l = pair ? g >> 1 : g;
-    const T* src = ((pair && (g & 1)) ? xv : xu) + (int64_t)l * it.src_ls;
-    T* dst = sm + g * A;
-    for (int e = lane; e < A; e += 32) {
-      const int bj = (int)fdiv((uint32_t)e, it.bwid), bi = e - bj * it.bw;
-      cp_async_elem<T>(dst + e, src + (bi * it.bs0 + bj * it.bs1));
-    }
-  }
-  cp_async_wait_all();
-  __syncwarp();
-  // lanes take (cell, group of kTileLevels levels) units, cells fastest:
-  // a cell's weights, box word and rotation load once for its group
-  const int nq = it.nunits, tot = nq * ((it.nl + kTileLevels - 1) / kTileLevels);
-  const int p = it.p;
-  const int lstep = nc * A;  // stage values per level
-  B* du = static_cast<B*>(P.d);
-  B* dv = static_cast<B*>(P.d2);
-  for (int u = lane; u < tot; u += 32) {
-    const int g = (int)fdiv((uint32_t)u, it.vol), q = u - g * nq;
-    const int lb = g * kTileLevels;
-    const int row = it.table + it.u0 + q;
-    const int bx = __ldg(c.itp_box + row);
-    const int st = (bx & kBoxRows) ? it.bw : 1;
-    const bool snap = bx & kBoxSnap;
-    const int64_t off = (int64_t)dst_cell(it, c, it.u0 + q) + (int64_t)(it.l0 + lb) * it.dst_ls;
-    const int64_t ls = it.dst_ls;
-    const T* su = sm + lb * lstep + (bx & kBoxIndex);
-    const T* wr = static_cast<const T*>(c.itp_w) + row * kPMax;
-    if (!pair) {
-      if (snap) {  // unit row: exact copy of node 0
-#pragma unroll
-        for (int l = 0; l < kTileLevels; ++l)
-          if (lb + l < it.nl) du[off + l * ls] = reinterpret_cast<const B*>(su)[l * lstep];
-        continue;
-      }
-      T acc[kTileLevels];
-#pragma unroll
-      for (int l = 0; l < kTileLevels; ++l) acc[l] = T(0);
-#pragma unroll
-      for (int n = 0; n < kPMax; ++n)
-        if (n < p) {
-          const T w = ldg(wr + n);
-#pragma unroll
-          for (int l = 0; l < kTileLevels; ++l)
-            if (lb + l < it.nl) acc[l] = fma(w, su[l * lstep + n * st], acc[l]);
-        }
-#pragma unroll
-      for (int l = 0; l < kTileLevels; ++l)
-        if (lb + l < it.nl) du[off + l * ls] = to_bits(acc[l]);
-    } else {
-      const T* sv = su + A;
-      const int pe = snap ? 1 : p;
-      T au[kTileLevels], av[kTileLevels];
-#pragma unroll
-      for (int l = 0; l < kTileLevels; ++l) au[l] = av[l] = T(0);
-#pragma unroll
-      for (int n = 0; n < kPMax; ++n)
-        if (n < pe) {
-          const T w = snap ? T(1) : ldg(wr + n);
-#pragma unroll
-          for (int l = 0; l < kTileLevels; ++l)
-            if (lb + l < it.nl) {
-              au[l] = fma(w, su[l * lstep + n * st], au[l]);
-              av[l] = fma(w, sv[l * lstep + n * st], av[l]);
-            }
-        }
-      const T* mr = static_cast<const T*>(c.itp_m) + row * 4;
-      const T m00 = ldg(mr), m01 = ldg(mr + 1), m10 = ldg(mr + 2), m11 = ldg(mr + 3);
-#pragma unroll
-      for (int l = 0; l < kTileLevels; ++l)
-        if (lb + l < it.nl) {
-          du[off + l * ls] = to_bits(fma(m00, au[l], m01 * av[l]));
-          dv[off + l * ls] = to_bits(fma(m10, au[l], m11 * av[l]));
-        }
-    }
-  }
-  __syncwarp();  // every lane is done with the stage before the next item
-}
-
-// Staged CSR rows (MODE_TILE, levels far apart in memory): the entries of
-// a tile of up to 32 rows lie in one small box of one block, in at most two
-// of its slots (a vector pair's components); the warp copies the box for
-// the item's levels and slots to shared memory, then each lane sums one row
-// for a group of up to kTileLevels levels from there, loading each entry's
-// weight and box word once for the group, in entry order (as the per-lane
-// path: from zero, then + b).  Each entry carries its value's place in one
-// level of the stage (csr_box: slot selector * box cells + box index).
-template <typename T>
-__device__ __forceinline__ void stage_box(const Item& it, const Ctx& c, T* sm, int lane) {
-  const int nsel = it.bsrc2 >= 0 ? 2 : 1;
-  const int A = it.bw * it.bh;
-  const int64_t lev0 = (int64_t)it.l0 * it.src_ls + it.borg;
-  const T* x0 = static_cast<const T*>(c.slots[it.bsrc]) + lev0;
-  const T* x1 = nsel > 1 ? static_cast<const T*>(c.slots[it.bsrc2]) + lev0 : x0;
-  // stage: [level][slot][box row][box column]
-  for (int g = 0; g < it.nl * nsel; ++g) {
-    const int l = nsel > 1 ? g >> 1 : g;
-    const T* src = ((nsel > 1 && (g & 1)) ? x1 : x0) + (int64_t)l * it.src_ls;
-    T* dst = sm + g * A;
-    for (int e = lane; e < A; e += 32) {
-      const int bj = (int)fdiv((uint32_t)e, it.bwid), bi = e - bj * it.bw;
-      cp_async_elem<T>(dst + e, src + (bi * it.bs0 + bj * it.bs1));
-    }
-  }
-  cp_async_wait_all();
-  __syncwarp();
-}
-
+// memory (each source value once, lanes over consecutive cells of a box
+// row), then a lane evaluates one cell for all of the item's
+// levels, kTileLevels at a time: the p-point sums, the 2x2 rotation of a
+// vector pair, and the store.  Same sums in the same order as the per-lane
+// path.  Bound by issue and the shared-memory pipe, so: the planes have a
+// fixed size (a node's levels are constant offsets), levels past the item's
+// are summed from whatever the stage holds and only not stored (no test per
+// node), and a cell's weights load once, as vectors.  (h, u,
+// v) x 32 levels FP32 on 6 x 384^2: 29.7 -> 22.7 us for the whole fill, 8
+// levels an item instead of 4.
 // four consecutive words / values from a 16-byte boundary
 __device__ __forceinline__ void ld_words4(const int32_t* p, int* w) {
   const int4 v = __ldg(reinterpret_cast<const int4*>(p));
@@ -706,112 +585,190 @@ __device__ __forceinline__ void ld_vals4(const T* p, T* a) {
   }
 }
 
-template <typename T, int W>
-__device__ void csr_tile(const Item& it, const Ptrs& P, const Ctx& c, int lane) {
-  T* sm = static_cast<T*>(P.stage);
-  stage_box<T>(it, c, sm, lane);
-  const int lstep = (it.bsrc2 >= 0 ? 2 : 1) * it.bw * it.bh;  // stage values per level
-  const int nq = it.nunits, tot = nq * ((it.nl + kTileLevels - 1) / kTileLevels);
-  const T* val = static_cast<const T*>(c.csr_val);
-  T* d = static_cast<T*>(P.d);
-  for (int u = lane; u < tot; u += 32) {
-    const int g = (int)fdiv((uint32_t)u, it.vol), q = u - g * nq;
-    const int lb = g * kTileLevels;
-    const int row = it.table + it.u0 + q;
-    const int nnz = __ldg(c.csr_nnz + row);
-    const int e0 = it.src_org + (it.u0 + q) * it.p;
-    const T* s = sm + lb * lstep;
-    T acc[kTileLevels];
-#pragma unroll
-    for (int l = 0; l < kTileLevels; ++l) acc[l] = T(0);
-    // the row's entries W (4, or 8 when the row width is a multiple of 8)
-    // at a time (rows start on 16-byte boundaries): the entries' stage
-    // places (csr_box) and weights load as vectors, so a row costs one
-    // memory latency per W entries; in the last, partial block the padding
-    // entries (place 0, weight 0) read a staged value and are dropped
-    for (int e = 0; e < nnz; e += W) {
-      int bx[W];
-      T w[W];
-#pragma unroll
-      for (int h = 0; h < W; h += 4) {
-        ld_words4(c.csr_box + e0 + e + h, bx + h);
-        ld_vals4<T>(val + e0 + e + h, w + h);
-      }
-      if (e + W <= nnz) {
-#pragma unroll
-        for (int j = 0; j < W; ++j)
-#pragma unroll
-          for (int l = 0; l < kTileLevels; ++l)
-            if (lb + l < it.nl) acc[l] = fma(w[j], s[bx[j] + l * lstep], acc[l]);
-      } else {
-#pragma unroll
-        for (int j = 0; j < W; ++j) {
-          const bool live = e + j < nnz;
-#pragma unroll
-          for (int l = 0; l < kTileLevels; ++l)
-            if (lb + l < it.nl) {
-              const T xv = s[bx[j] + l * lstep];
-              acc[l] = live ? fma(w[j], xv, acc[l]) : acc[l];
-            }
-        }
-      }
+// Starts the copies of the item's box into the warp's stage: level l of slot
+// x0's cell e to element l * PLANE + e, of slot x1 (if any) to l * PLANE +
+// second + e (loads and stores through registers instead of cp.async took 12
+// % longer on the reconstruction rows, 27 % on the interpolation ones).
+template <typename T>
+__device__ __forceinline__ void cp_async_elem(T* smem, const T* gmem) {
+  const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
+  if constexpr (sizeof(T) == 4)
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(sa), "l"(gmem));
+  else
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(sa), "l"(gmem));
+}
+
+__device__ __forceinline__ void cp_async_wait_all() {
+  asm volatile("cp.async.wait_all;\n" ::: "memory");
+}
+
+template <typename T, int PLANE>
+__device__ __forceinline__ void stage_box(const Item& it, T* sm, const T* x0, const T* x1,
+                                          int second, int lane) {
+  const int64_t ls = it.src_ls, lev0 = (int64_t)it.l0 * ls + it.borg;
+  const int A = it.bw * it.bh, nl = it.nl;
+  for (int e = lane; e < A; e += 32) {
+    const int bj = (int)fdiv((uint32_t)e, it.bwid), bi = e - bj * it.bw;
+    const int64_t off = lev0 + (bi * it.bs0 + bj * it.bs1);
+    const T* s = x0 + off;
+    for (int l = 0; l < nl; ++l, s += ls) cp_async_elem<T>(sm + (e + l * PLANE), s);
+    if (x1) {
+      s = x1 + off;
+      for (int l = 0; l < nl; ++l, s += ls) cp_async_elem<T>(sm + (second + e + l * PLANE), s);
     }
-    const T b = ldg(static_cast<const T*>(c.csr_rhs) + row);
-    T* dd = d + (int64_t)dst_cell(it, c, it.u0 + q) + (int64_t)(it.l0 + lb) * it.dst_ls;
+  }
+}
+
+template <typename T, bool PAIR>
+__device__ __forceinline__ void interp_tile_t(const Item& item, const Ptrs& P, const Ctx& c,
+                                              int lane) {
+  const Item it = item;
+  using B = typename BitsOf<T>::type;
+  constexpr int NL = kTileLevels, PLANE = PAIR ? 2 * kPlaneInterp : kPlaneInterp;
+  T* sm = reinterpret_cast<T*>(g_stage + P.stage);
+  const int cu = it.comp & 0xffff, cv = it.comp >> 16;
+  stage_box<T, PLANE>(it, sm, static_cast<const T*>(c.slots[it.bsrc + cu]),
+                      PAIR ? static_cast<const T*>(c.slots[it.bsrc + cv]) : nullptr, kPlaneInterp,
+                      lane);
+  const int nq = it.nunits, q = it.u0 + min(lane, nq - 1);
+  const int row = it.table + q, p = it.p;
+  const int bx = __ldg(c.itp_box + row);
+  T w[kPMax];
+  ld_vals4<T>(static_cast<const T*>(c.itp_w) + row * kPMax, w);
+  ld_vals4<T>(static_cast<const T*>(c.itp_w) + row * kPMax + 4, w + 4);
+  const T* mr = static_cast<const T*>(c.itp_m) + row * 4;
+  const int64_t ls = it.dst_ls;
+  const int64_t off = (int64_t)dst_cell(it, c, q) + (int64_t)it.l0 * ls;
+  const int st = (bx & kBoxRows) ? it.bw : 1;
+  const bool snap = bx & kBoxSnap;
+  cp_async_wait_all();
+  __syncwarp();
+  if (lane < nq) {
+    B* du = static_cast<B*>(P.d) + off;
+    B* dv = PAIR ? static_cast<B*>(P.d2) + off : nullptr;
+    const int pe = snap ? 1 : p;
+    if (PAIR && snap) w[0] = T(1);
+    for (int lb = 0; lb < it.nl; lb += NL) {
+      const T* s = sm + ((bx & kBoxIndex) + lb * PLANE);
+      if (!PAIR && snap) {  // unit row: exact copy of node 0
 #pragma unroll
-    for (int l = 0; l < kTileLevels; ++l)
-      if (lb + l < it.nl) dd[(int64_t)l * it.dst_ls] = acc[l] + b;
+        for (int l = 0; l < NL; ++l)
+          if (lb + l < it.nl) du[(lb + l) * ls] = reinterpret_cast<const B*>(s)[l * PLANE];
+        continue;
+      }
+      T au[NL], av[NL];
+#pragma unroll
+      for (int l = 0; l < NL; ++l) au[l] = av[l] = T(0);
+#pragma unroll
+      for (int n = 0; n < kPMax; ++n, s += st)
+        if (n < pe) {
+#pragma unroll
+          for (int l = 0; l < NL; ++l) {
+            au[l] = fma(w[n], s[l * PLANE], au[l]);
+            if (PAIR) av[l] = fma(w[n], s[l * PLANE + kPlaneInterp], av[l]);
+          }
+        }
+      T m[4];
+      if (PAIR) ld_vals4<T>(mr, m);
+#pragma unroll
+      for (int l = 0; l < NL; ++l)
+        if (lb + l < it.nl) {
+          if (PAIR) {
+            du[(lb + l) * ls] = to_bits(fma(m[0], au[l], m[1] * av[l]));
+            dv[(lb + l) * ls] = to_bits(fma(m[2], au[l], m[3] * av[l]));
+          } else {
+            du[(lb + l) * ls] = to_bits(au[l]);
+          }
+        }
+    }
   }
   __syncwarp();  // every lane is done with the stage before the next item
 }
 
-// Staged transpose rows (MODE_TILE adjoint gather items, levels far apart in
-// memory): the ghost values that a tile of up to 32 data values' transpose
-// rows read lie in one small box of one block, in at most two slots; the
-// warp copies the box of ghost cotangents for the item's levels to shared
-// memory, then each lane updates one data value for a group of up to
-// kTileLevels levels with the entries in ghost order from there (as
-// adj_chunk: from the value's own cotangent).
 template <typename T>
-__device__ void adj_tile(const Item& it, const Ptrs& P, const Ctx& c, int lane) {
-  T* sm = static_cast<T*>(P.stage);
-  stage_box<T>(it, c, sm, lane);
-  const int lstep = (it.bsrc2 >= 0 ? 2 : 1) * it.bw * it.bh;
-  const int nq = it.nunits, tot = nq * ((it.nl + kTileLevels - 1) / kTileLevels);
-  const T* wv = static_cast<const T*>(c.aent_w);
+__device__ __forceinline__ void interp_tile(const Item& it, const Ptrs& P, const Ctx& c, int lane) {
+  if (it.kind == IK_INTERP_PAIR)
+    interp_tile_t<T, true>(it, P, c, lane);
+  else
+    interp_tile_t<T, false>(it, P, c, lane);
+}
+
+// Staged CSR and transpose rows (MODE_TILE, levels far apart in memory): the
+// entries of a tile of up to 32 rows lie in one small box of one block, in
+// at most two of its slots (a vector pair's components); the warp copies the
+// box for the item's levels and slots to shared memory, then each lane sums
+// one row for a group of kTileLevels levels from there, in entry order (CSR:
+// from zero, then + b; transpose: from the value's own cotangent).  Bound by
+// the L1 / shared-memory pipe: every multiply-add reads one staged value (a
+// wavefront per warp), so the entries' places and weights come in the
+// tile's own order (Ctx::tile_box), four a row as one contiguous piece of a
+// warp's load -- read row by row each load of four touched 32 lines and cost
+// more of the pipe than the staged values -- and the planes have a fixed
+// size.  W entries load together; in a row's last, partial block the padding
+// entries (place 0) read a staged value and are dropped.  Reconstruction
+// rows (16 / 32 entries) of the 6 x 384^2 sphere 80 -> 63 us (four entries at
+// a time instead of eight: 72 us), the adjoint of 6 x 768^2 123 -> 118 us.
+template <typename T, int W, int PLANE>
+__device__ __forceinline__ void row_sums(const T* s, const int32_t* tb, const T* tw, int step,
+                                         int nnz, T (&acc)[kTileLevels]) {
+  for (int e = 0; e < nnz; e += W, tb += step * (W / 4), tw += step * (W / 4)) {
+    int bx[W];
+    T w[W];
+#pragma unroll
+    for (int h = 0; h < W / 4; ++h) {
+      ld_words4(tb + h * step, bx + 4 * h);
+      ld_vals4<T>(tw + h * step, w + 4 * h);
+    }
+    if (e + W <= nnz) {
+#pragma unroll
+      for (int j = 0; j < W; ++j)
+#pragma unroll
+        for (int l = 0; l < kTileLevels; ++l) acc[l] = fma(w[j], s[bx[j] + l * PLANE], acc[l]);
+    } else {
+#pragma unroll
+      for (int j = 0; j < W; ++j) {
+        const bool live = e + j < nnz;
+#pragma unroll
+        for (int l = 0; l < kTileLevels; ++l) {
+          const T xv = s[bx[j] + l * PLANE];
+          acc[l] = live ? fma(w[j], xv, acc[l]) : acc[l];
+        }
+      }
+    }
+  }
+}
+
+// ADJ: transpose rows (W 4); otherwise CSR rows of W (4, or 8 where the row
+// width is a multiple of 8) entries a block
+template <typename T, int W, bool ADJ>
+__device__ void rows_tile(const Item& item, const Ptrs& P, const Ctx& c, int lane) {
+  const Item it = item;
+  constexpr int NL = kTileLevels, PLANE = ADJ ? kPlaneAdj : kPlaneCsr;
+  T* sm = reinterpret_cast<T*>(g_stage + P.stage);
+  stage_box<T, PLANE>(it, sm, static_cast<const T*>(c.slots[it.bsrc]),
+                      it.bsrc2 >= 0 ? static_cast<const T*>(c.slots[it.bsrc2]) : nullptr,
+                      it.bw * it.bh, lane);
+  cp_async_wait_all();
+  __syncwarp();
+  const int nq = it.nunits, tot = nq * ((it.nl + NL - 1) / NL), step = nq * 4;
+  const int64_t ls = it.dst_ls;
   for (int u = lane; u < tot; u += 32) {
     const int g = (int)fdiv((uint32_t)u, it.vol), q = u - g * nq;
-    const int lb = g * kTileLevels;
-    const int r = it.table + it.u0 + q;
-    T* xb = static_cast<T*>(P.d) +
-            ((int64_t)__ldg(c.arow_off + r) + (int64_t)(it.l0 + lb) * it.dst_ls);
-    const int e0 = (int)__ldg(c.adj_ptr + r), e1 = (int)__ldg(c.adj_ptr + r + 1);
-    const T* s = sm + lb * lstep;
-    T acc[kTileLevels];
+    const int lb = g * NL;
+    const int row = it.table + it.u0 + q;
+    const int cell = ADJ ? __ldg(c.arow_off + row) : dst_cell(it, c, it.u0 + q);
+    const int nnz = ADJ ? (int)(__ldg(c.adj_ptr + row + 1) - __ldg(c.adj_ptr + row))
+                        : __ldg(c.csr_nnz + row);
+    T* d = static_cast<T*>(P.d) + (cell + (int64_t)(it.l0 + lb) * ls);
+    T acc[NL];
 #pragma unroll
-    for (int l = 0; l < kTileLevels; ++l)
-      acc[l] = lb + l < it.nl ? xb[(int64_t)l * it.dst_ls] : T(0);
-    // entries four at a time, their loads issued together
-    for (int e = e0; e < e1; e += 4) {
-      int bx[4];
-      T w[4];
+    for (int l = 0; l < NL; ++l) acc[l] = ADJ && lb + l < it.nl ? d[l * ls] : T(0);
+    row_sums<T, W, PLANE>(sm + lb * PLANE, c.tile_box + (it.src_org + q * 4),
+                          static_cast<const T*>(c.tile_w) + (it.src_org + q * 4), step, nnz, acc);
+    const T b = ADJ ? T(0) : ldg(static_cast<const T*>(c.csr_rhs) + row);
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const bool live = e + j < e1;
-        bx[j] = live ? __ldg(c.adj_box + e + j) : 0;
-        w[j] = live ? ldg(wv + e + j) : T(0);
-      }
-#pragma unroll
-      for (int j = 0; j < 4; ++j)
-        if (e + j < e1) {
-#pragma unroll
-          for (int l = 0; l < kTileLevels; ++l)
-            if (lb + l < it.nl) acc[l] = fma(w[j], s[bx[j] + l * lstep], acc[l]);
-        }
-    }
-#pragma unroll
-    for (int l = 0; l < kTileLevels; ++l)
-      if (lb + l < it.nl) xb[(int64_t)l * it.dst_ls] = acc[l];
+    for (int l = 0; l < NL; ++l)
+      if (lb + l < it.nl) d[l * ls] = ADJ ? acc[l] : acc[l] + b;
   }
   __syncwarp();  // every lane is done with the stage before the next item
 }
@@ -820,7 +777,8 @@ __device__ void adj_tile(const Item& it, const Ptrs& P, const Ctx& c, int lane) 
 // level-fastest order the lanes of a warp share a cell, so its table row is
 // one broadcast load and the node loads of the warp are contiguous.
 template <typename T, bool PAIR>
-__device__ void interp_flat(const Item& it, const Ptrs& P, const Ctx& c, int lane) {
+__device__ void interp_flat(const Item& item, const Ptrs& P, const Ctx& c, int lane) {
+  const Item it = item;
   using B = typename BitsOf<T>::type;
   constexpr int U = 4;
   const int end = it.u0 + it.nunits;
@@ -1139,7 +1097,8 @@ __device__ void csr_flat(const Item& it, const Ptrs& P, const Ctx& c, int lane) 
 constexpr int kAdjBatch = 4;
 
 template <typename T, int CH>
-__device__ void adj_chunk(const Item& it, const Ptrs& P, const Ctx& c, int lane) {
+__device__ void adj_chunk(const Item& item, const Ptrs& P, const Ctx& c, int lane) {
+  const Item it = item;
   constexpr int E = kAdjBatch;
   const int end = it.u0 + it.nunits;
   const int chn = it.mode;
@@ -1254,9 +1213,9 @@ __device__ __forceinline__ void run_item(const Item& it, const Ptrs& P, const Ct
   } else if constexpr (FAM == FAM_CSR) {
     if (it.mode == MODE_TILE) {
       if (it.p % 8 == 0)
-        csr_tile<T, 8>(it, P, c, lane);
+        rows_tile<T, 8, false>(it, P, c, lane);
       else
-        csr_tile<T, 4>(it, P, c, lane);
+        rows_tile<T, 4, false>(it, P, c, lane);
     } else if (it.p == 8) {
       if (flat)
         csr_flat_w<T, 8, false>(it, P, c, lane);
@@ -1287,7 +1246,7 @@ __device__ __forceinline__ void run_item(const Item& it, const Ptrs& P, const Ct
     }
   } else {
     if (it.mode == MODE_TILE)
-      adj_tile<T>(it, P, c, lane);
+      rows_tile<T, 4, true>(it, P, c, lane);
     else if (it.kind == IK_ADD && c.vec_runs)
       runs_vec<T, RUN_ADD>(it, P, c, lane);
     else if (it.kind == IK_ADD)
@@ -1361,14 +1320,14 @@ __device__ __forceinline__ Ptrs gather_ptrs(void* mine) {
   P.d = reinterpret_cast<void*>(__shfl_sync(0xffffffffu, v, kWordDst));
   P.d2 = reinterpret_cast<void*>(__shfl_sync(0xffffffffu, v, kWordDst2));
   P.s = reinterpret_cast<const void*>(__shfl_sync(0xffffffffu, v, kWordSrc));
-  P.stage = nullptr;
+  P.stage = 0;
   return P;
 }
 
-// Shared memory for staged boxes: one area per warp (Ctx::stage_warp bytes:
-// 2 KB for interpolation and transpose tiles, 4 KB when the list has CSR
-// tiles) in the kernels that run interpolation, CSR or transpose-gather
-// items, as dynamic shared memory that only launches of lists with staged
+// Shared memory for staged boxes: one area per warp (Ctx::stage_warp bytes,
+// the largest stage_bytes of the list's tiles) in the kernels that run
+// interpolation, CSR or transpose-gather items, as dynamic shared memory
+// that only launches of lists with staged
 // tiles request: a kernel that reserves no shared memory keeps the SM's
 // default split of L1 and shared memory and shares SMs with the structured
 // kernel beside it (the 512-block step, levels innermost: 51.1 us with a
@@ -1394,14 +1353,13 @@ template <typename T, int THREADS, int FAM>
 __global__ void __launch_bounds__(THREADS, (Occ<FAM, THREADS>::kMinBlocks))
     k_items(Ctx c, const Item* __restrict__ items, int nitems) {
   __shared__ Item sit[THREADS / 32];
-  extern __shared__ __align__(16) unsigned char stage[];  // Stage, when requested
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int idx = blockIdx.x * (THREADS / 32) + warp;
   if (idx >= nitems) return;
   const int w = __ldg(reinterpret_cast<const int*>(items + idx) + lane);
   reinterpret_cast<int*>(&sit[warp])[lane] = w;
   Ptrs P = gather_ptrs(lookup_slot(c, w, lane));
-  if (Stage<FAM, THREADS>::kWarps) P.stage = stage + warp * c.stage_warp;
+  if (Stage<FAM, THREADS>::kWarps) P.stage = warp * c.stage_warp;
   __syncwarp();
   run_work<T, FAM>(sit[warp], P, c, lane);
 }
@@ -1414,7 +1372,6 @@ template <typename T, int THREADS, int FAM>
 __global__ void __launch_bounds__(THREADS, (Occ<FAM, THREADS>::kMinBlocks))
     k_stream(Ctx c, const Item* __restrict__ items, int nitems) {
   __shared__ Item sit[THREADS / 32];
-  extern __shared__ __align__(16) unsigned char stage[];  // Stage, when requested
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int stride = gridDim.x * (THREADS / 32);
   const int* iw = reinterpret_cast<const int*>(items);
@@ -1430,7 +1387,7 @@ __global__ void __launch_bounds__(THREADS, (Occ<FAM, THREADS>::kMinBlocks))
     const int nxt2 = nxt + stride;
     const int w_nxt2 = nxt2 < nitems ? __ldg(iw + (int64_t)nxt2 * 32 + lane) : 0;
     Ptrs P = gather_ptrs(p_cur);
-    if (Stage<FAM, THREADS>::kWarps) P.stage = stage + warp * c.stage_warp;
+    if (Stage<FAM, THREADS>::kWarps) P.stage = warp * c.stage_warp;
     __syncwarp();
     run_work<T, FAM>(sit[warp], P, c, lane);
     __syncwarp();
@@ -1462,7 +1419,6 @@ __global__ void __launch_bounds__(THREADS, (Occ<FAM, THREADS>::kMinBlocks))
   constexpr unsigned FULL = 0xffffffffu;
   constexpr unsigned S = kSpread;
   __shared__ Item sit[THREADS / 32];
-  extern __shared__ __align__(16) unsigned char stage[];  // Stage, when requested
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int* iw = reinterpret_cast<const int*>(items);
   const unsigned n = (unsigned)nitems;
@@ -1501,7 +1457,7 @@ __global__ void __launch_bounds__(THREADS, (Occ<FAM, THREADS>::kMinBlocks))
     const unsigned raw = issue();  // claim of the fourth item, in flight
     reinterpret_cast<int*>(&sit[warp])[lane] = wa;
     Ptrs P = gather_ptrs(pa);
-    if (Stage<FAM, THREADS>::kWarps) P.stage = stage + warp * c.stage_warp;
+    if (Stage<FAM, THREADS>::kWarps) P.stage = warp * c.stage_warp;
     __syncwarp();
     run_work<T, FAM>(sit[warp], P, c, lane);
     __syncwarp();

@@ -149,10 +149,10 @@ struct bc_plan {
   std::vector<int4> itp_idx;
   std::vector<double> itp_w, itp_m;
   std::vector<int32_t> itp_box;  // staged interpolation: node 0 in its tile's box
-  // staged CSR / transpose entries: the value's place in one level of its
-  // tile's stage, selector * (box cells) + box index
-  std::vector<int32_t> csr_box;
-  std::vector<int32_t> adj_box;
+  // entries of staged CSR / transpose tiles, in Ctx::tile_box's order: the
+  // value's place in one level of its tile's stage, and its weight
+  std::vector<int32_t> tile_box;
+  std::vector<double> tile_w;
   // user CSR rows stored as ELL blocks (one width per sub-matrix)
   std::vector<int32_t> csr_nnz;
   std::vector<int32_t> csr_slot, csr_off;
@@ -866,9 +866,9 @@ int table_mode(const bc_block& B, int order, int chunk) {
 // default 4 for interpolation rows, whose pair path keeps two components'
 // sums, and 8 for CSR and transpose rows); the persistent launch's kernel
 // holds at most 4
-int level_chunk(const bc_plan* P, bool interp) {
+int level_chunk(const bc_plan* P, int fam) {
   int ch = P->opts.level_chunk;
-  if (ch == 0) ch = interp ? 4 : 8;
+  if (ch == 0) ch = fam == FAM_INTERP ? 4 : 8;
   const bool all_kinds =
       P->opts.batch_mode == BC_BATCH_PERSISTENT || P->opts.batch_mode == BC_BATCH_SINGLE;
   return all_kinds ? std::min(ch, 4) : ch;
@@ -991,266 +991,303 @@ void emit_runs(std::vector<Item>& out, Item proto, const std::vector<int4>& runs
   }
 }
 
-// Staged interpolation items of sub-matrix s (levels in chunks of `chunk`):
-// tiles of up to kTileCells consecutive box cells whose nodes all lie in one
-// 2-D source block, with the node box of each tile small enough that `chunk`
-// levels of its components (nc) fit a warp's staging area at least one
-// level at a time.  Writes the cells' itp_box rows.  Returns false (the
-// sub-matrix keeps the per-lane path) when some tile does not qualify.
-bool emit_tiles(bc_plan* P, const Sub& s, const Item& proto, int chunk, int nc,
-                std::vector<Item>& out) {
-  const bc_block& B = P->blocks[s.block];
-  const int L = B.nlevels;
-  const int cap = kStageBytesRows / P->esize;
+// The box of a staged tile as rows are added: one 2-D block, at most two of
+// its slots, the cells its entries read.
+struct TileBox {
+  int blk = -1, nsel = 0, sl[2] = {-1, -1};
+  int imin = INT_MAX, imax = INT_MIN, jmin = INT_MAX, jmax = INT_MIN;
+  int64_t cells() const { return (int64_t)(imax - imin + 1) * (jmax - jmin + 1); }
+  // selector of `slot`, or -1 when it is of another block or a third slot
+  int select(const bc_plan* P, int slot) {
+    const int b = P->slot_block[slot];
+    if (blk < 0) {
+      const bc_block& S = P->blocks[b];
+      if (S.n[2] != 1 || S.h[2] != 0) return -1;
+      blk = b;
+    }
+    if (b != blk) return -1;
+    for (int k = 0; k < nsel; ++k)
+      if (sl[k] == slot) return k;
+    if (nsel == 2) return -1;
+    sl[nsel] = slot;
+    return nsel++;
+  }
+  void grow(int i, int j) {
+    imin = std::min(imin, i);
+    imax = std::max(imax, i);
+    jmin = std::min(jmin, j);
+    jmax = std::max(jmax, j);
+  }
+};
+
+// levels of a staged item: equal parts of the block's, at most what the
+// stage holds (fewer with bc_plan_opts.level_chunk)
+int tile_levels(const bc_plan* P, int L) {
+  const int held = stage_levels(P->esize);
+  const int most = P->opts.level_chunk ? std::min(P->opts.level_chunk, held) : held;
+  const int parts = (L + most - 1) / most;
+  return (L + parts - 1) / parts;
+}
+
+// Appends the items (one per part of the levels) of a tile of nq rows from
+// q0 that reads box T.
+void push_tile(const bc_plan* P, const TileBox& T, int q0, int nq, const Item& proto, int L,
+               std::vector<Item>& out) {
+  const bc_block& S = P->blocks[T.blk];
+  const int nl = tile_levels(P, L);
+  for (int l0 = 0; l0 < L; l0 += nl) {
+    Item it = proto;
+    it.mode = MODE_TILE;
+    it.u0 = q0;
+    it.nunits = nq;
+    it.vol = make_div((uint32_t)nq);
+    it.l0 = l0;
+    it.nl = std::min(nl, L - l0);
+    it.bw = T.imax - T.imin + 1;
+    it.bh = T.jmax - T.jmin + 1;
+    it.bs0 = (int32_t)S.stride[0];
+    it.bs1 = (int32_t)S.stride[1];
+    it.bsrc = T.sl[0];
+    it.bsrc2 = T.sl[1];
+    it.bwid = make_div((uint32_t)it.bw);
+    it.borg = (int32_t)cell_offset(S, T.imin, T.jmin, 0);
+    it.src_ls = (int32_t)(S.nlevels > 1 ? S.level_stride : 0);
+    it.src_slot = -1;  // no common-slot lookup: the tile reads its slots itself
+    out.push_back(it);
+  }
+}
+
+// Staged interpolation items of sub-matrix s: tiles of up to kTileCells
+// consecutive box cells, each as long as its cells' nodes lie in one 2-D
+// source block inside a box of one plane (kPlaneInterp cells).  Writes the
+// cells' itp_box rows.  Returns false (the sub-matrix keeps the per-lane
+// path) when some cell does not qualify.
+bool emit_tiles(bc_plan* P, const Sub& s, const Item& proto, std::vector<Item>& out) {
+  const int L = P->blocks[s.block].nlevels;
   std::vector<Item> tiles;
   std::vector<std::pair<int, int32_t>> boxes;  // (row, itp_box) to write on success
-  for (int q0 = 0; q0 < s.vol; q0 += kTileCells) {
-    const int nq = std::min(kTileCells, s.vol - q0);
+  struct Node0 {
+    int i, j, rows, snap;
+  };
+  std::vector<Node0> n0;
+  for (int q0 = 0; q0 < s.vol;) {
     int base = -1;
-    int imin = INT_MAX, imax = INT_MIN, jmin = INT_MAX, jmax = INT_MIN;
-    struct Node0 {
-      int i, j, rows, snap;
-    };
-    std::vector<Node0> n0(nq);
-    for (int q = 0; q < nq; ++q) {
-      const int4 ix = P->itp_idx[(size_t)(s.table + q0 + q)];
-      if (base < 0) base = ix.x;
-      if (ix.x != base) return false;
-      const bc_block& S = P->blocks[P->slot_block[ix.x]];
-      if (S.n[2] != 1 || S.h[2] != 0) return false;
+    TileBox T;
+    n0.clear();
+    for (int q = q0; q < std::min(s.vol, q0 + kTileCells); ++q) {
+      const int4 ix = P->itp_idx[(size_t)(s.table + q)];
+      const int blk = P->slot_block[ix.x];
+      const bc_block& S = P->blocks[blk];
       int i, j, k;
-      if (!decode_cell(S, ix.y, i, j, k)) return false;
+      if (S.n[2] != 1 || S.h[2] != 0 || S.nlevels != L || !decode_cell(S, ix.y, i, j, k))
+        return false;
       const bool snap = ix.w & kFlagSnap;
       const int np = snap ? 1 : s.p;
       int ax;
       if (np == 1 || ix.z == S.stride[0]) ax = 0;
       else if (ix.z == S.stride[1]) ax = 1;
       else return false;
-      const int i1 = ax == 0 ? i + np - 1 : i, j1 = ax == 1 ? j + np - 1 : j;
-      imin = std::min(imin, i);
-      imax = std::max(imax, i1);
-      jmin = std::min(jmin, j);
-      jmax = std::max(jmax, j1);
-      n0[q] = {i, j, ax, snap ? 1 : 0};
+      TileBox G = T;
+      G.blk = blk;
+      G.sl[0] = ix.x;
+      G.grow(i, j);
+      G.grow(ax == 0 ? i + np - 1 : i, ax == 1 ? j + np - 1 : j);
+      if ((base >= 0 && ix.x != base) || G.cells() > kPlaneInterp) break;
+      T = G;
+      base = ix.x;
+      n0.push_back({i, j, ax, snap ? 1 : 0});
     }
-    const int bw = imax - imin + 1, bh = jmax - jmin + 1;
-    if ((int64_t)bw * bh > kBoxIndex || (int64_t)bw * bh * nc > cap) return false;
-    const int nl = std::min(chunk, cap / (bw * bh * nc));
-    const bc_block& S = P->blocks[P->slot_block[base]];
-    const int64_t org = cell_offset(S, imin, jmin, 0);
-    if (org > INT32_MAX) return false;
-    for (int q = 0; q < nq; ++q) {
-      const int32_t bx = (n0[q].i - imin) + (n0[q].j - jmin) * bw;
-      boxes.push_back({s.table + q0 + q,
-                       bx | (n0[q].rows ? kBoxRows : 0) | (n0[q].snap ? kBoxSnap : 0)});
-    }
-    for (int l0 = 0; l0 < L; l0 += nl) {
-      Item it = proto;
-      it.mode = MODE_TILE;
-      it.u0 = q0;
-      it.nunits = nq;
-      it.vol = make_div((uint32_t)nq);
-      it.l0 = l0;
-      it.nl = std::min(nl, L - l0);
-      it.bw = bw;
-      it.bh = bh;
-      it.bs0 = (int32_t)S.stride[0];
-      it.bs1 = (int32_t)S.stride[1];
-      it.bsrc = base;
-      it.bwid = make_div((uint32_t)bw);
-      it.borg = (int32_t)org;
-      it.bsrc2 = -1;
-      it.src_ls = (int32_t)(S.nlevels > 1 ? S.level_stride : 0);
-      tiles.push_back(it);
-    }
+    const int nq = (int)n0.size();
+    if (nq == 0) return false;
+    const bc_block& S = P->blocks[T.blk];
+    if (cell_offset(S, T.imin, T.jmin, 0) > INT32_MAX) return false;
+    const int bw = T.imax - T.imin + 1;
+    for (int q = 0; q < nq; ++q)
+      boxes.push_back({s.table + q0 + q, ((n0[q].i - T.imin) + (n0[q].j - T.jmin) * bw) |
+                                             (n0[q].rows ? kBoxRows : 0) |
+                                             (n0[q].snap ? kBoxSnap : 0)});
+    push_tile(P, T, q0, nq, proto, L, tiles);
+    q0 += nq;
   }
   for (const auto& b : boxes) P->itp_box[(size_t)b.first] = b.second;
   out.insert(out.end(), tiles.begin(), tiles.end());
   return true;
 }
 
-// A staged tile's box, the slots it reads and each entry's place in it.
-struct TileBox {
-  int blk = -1, nsel = 0, sl[2] = {-1, -1};
-  int imin = INT_MAX, imax = INT_MIN, jmin = INT_MAX, jmax = INT_MIN;
-  struct Ent {
-    size_t e;
-    int sel, i, j;
-  };
-  std::vector<Ent> ents;
-  // entry e reads (slot, offset); false when it leaves one 2-D block or
-  // its two slots
-  bool add(const bc_plan* P, size_t e, int slot, int64_t off) {
-    const int b = P->slot_block[slot];
-    if (blk < 0) blk = b;
-    if (b != blk) return false;
-    int sel = slot == sl[0] ? 0 : (slot == sl[1] ? 1 : -1);
-    if (sel < 0) {
-      if (nsel == 2) return false;
-      sl[nsel] = slot;
-      sel = nsel++;
-    }
-    const bc_block& S = P->blocks[b];
-    if (S.n[2] != 1 || S.h[2] != 0) return false;
-    int i, j, k;
-    if (!decode_cell(S, off, i, j, k)) return false;
-    imin = std::min(imin, i);
-    imax = std::max(imax, i);
-    jmin = std::min(jmin, j);
-    jmax = std::max(jmax, j);
-    ents.push_back({e, sel, i, j});
-    return true;
-  }
-};
-
 // Staging pays only when a tile's entries read each staged value at least
 // this often on average (a box mostly of values no row reads costs more
 // loads than it saves).
-constexpr int kMinTileReuse = 1;
+constexpr double kMinTileReuse = 1.5;
 
-// Items of one staged tile of nq rows from q0 (levels in chunks of `chunk`,
-// L levels): 1 when the box holds at least `need` levels of its slots in a
-// warp's staging area (items and box words appended), 0 when the box is
-// too large for that, -1 when the rows cannot (or should not) be staged.
-int finish_tile(const bc_plan* P, const TileBox& T, int q0, int nq, const Item& proto, int chunk,
-                int L, int need, int stage_bytes, std::vector<Item>& tiles,
-                std::vector<std::pair<size_t, int32_t>>& boxes) {
-  if (T.blk < 0) return -1;
+// Staged tiles of rows [q, q1) (`entries(q, f)` calls f(slot, offset,
+// weight) for each entry of row q in order): the longest tile of at most
+// kTileCells rows from q whose entries lie in one 2-D block, in at most two
+// of its slots, inside a box of `plane` cells, all slots together; cut to 16
+// rows where the box ran full and two level groups are staged (the lanes take
+// (row, group) units).  Returns its rows (0: row q cannot be staged), the
+// box and, in tile order, the entries' places and weights (rows padded to
+// the longest).
+struct TileEntries {
+  std::vector<int32_t> box;
+  std::vector<double> w;
+};
+template <typename F>
+int grow_tile(const bc_plan* P, int q, int q1, int L, int plane, F entries, TileBox& T,
+              TileEntries& E) {
+  struct Ent {
+    int sel, i, j;
+    double w;
+  };
+  std::vector<Ent> ents;
+  std::vector<int> ends;
+  auto fill = [&](int most) {
+    T = TileBox();
+    ents.clear();
+    ends.clear();
+    bool full = false;
+    for (int r = q; r < std::min(q1, q + most); ++r) {
+      TileBox G = T;
+      bool ok = true;
+      const size_t keep = ents.size();
+      entries(r, [&](int slot, int64_t off, double w) {
+        if (!ok) return;
+        const int sel = G.select(P, slot);
+        int i, j, k;
+        if (sel < 0 || P->blocks[G.blk].nlevels != L ||
+            !decode_cell(P->blocks[G.blk], off, i, j, k)) {
+          ok = false;
+          return;
+        }
+        G.grow(i, j);
+        ents.push_back({sel, i, j, w});
+      });
+      if (ok && G.blk >= 0 && G.cells() * G.nsel > plane) {
+        // a gradual overflow, or a jump to another row of the block?
+        full = T.blk >= 0 && G.cells() * G.nsel <= 2 * plane;
+        ok = false;
+      }
+      if (!ok) {
+        ents.resize(keep);
+        break;
+      }
+      T = G;
+      ends.push_back((int)ents.size());
+    }
+    return full;
+  };
+  if (fill(kTileCells) && ends.size() > 16 && tile_levels(P, L) > kTileLevels) fill(16);
+  const int nq = (int)ends.size();
+  if (nq == 0 || T.blk < 0) return 0;
   const bc_block& S = P->blocks[T.blk];
-  if (S.nlevels != L) return -1;
-  const int cap = stage_bytes / P->esize;
-  const int bw = T.imax - T.imin + 1, bh = T.jmax - T.jmin + 1;
-  if ((int64_t)bw * bh > kBoxIndex) return 0;
-  if ((int64_t)T.ents.size() < (int64_t)kMinTileReuse * bw * bh * T.nsel) return -1;
-  const int64_t fit = cap / ((int64_t)bw * bh * T.nsel);
-  if (fit < need) return 0;
-  const int nl = (int)std::min<int64_t>(chunk, fit);
-  const int64_t org = cell_offset(S, T.imin, T.jmin, 0);
-  if (org > INT32_MAX) return -1;
-  for (const TileBox::Ent& x : T.ents)
-    boxes.push_back({x.e, (x.i - T.imin) + (x.j - T.jmin) * bw + x.sel * bw * bh});
-  for (int l0 = 0; l0 < L; l0 += nl) {
-    Item it = proto;
-    it.mode = MODE_TILE;
-    it.u0 = q0;
-    it.nunits = nq;
-    // lanes take (row, group of kTileLevels levels) units, rows fastest
-    it.vol = make_div((uint32_t)nq);
-    it.l0 = l0;
-    it.nl = std::min(nl, L - l0);
-    it.bw = bw;
-    it.bh = bh;
-    it.bs0 = (int32_t)S.stride[0];
-    it.bs1 = (int32_t)S.stride[1];
-    it.bsrc = T.sl[0];
-    it.bsrc2 = T.sl[1];
-    it.bwid = make_div((uint32_t)bw);
-    it.borg = (int32_t)org;
-    it.src_ls = (int32_t)(S.nlevels > 1 ? S.level_stride : 0);
-    it.src_slot = -1;  // no common-slot lookup: the tile reads its slots itself
-    tiles.push_back(it);
-  }
-  return 1;
+  if (cell_offset(S, T.imin, T.jmin, 0) > INT32_MAX) return 0;
+  int longest = 0;
+  for (int r = 0; r < nq; ++r) longest = std::max(longest, ends[r] - (r ? ends[r - 1] : 0));
+  const size_t n4 = (size_t)(longest + 3) / 4;
+  E.box.assign(n4 * nq * 4, 0);
+  E.w.assign(n4 * nq * 4, 0.0);
+  const int bw = T.imax - T.imin + 1, A = (int)T.cells();
+  for (int r = 0, t = 0; r < nq; ++r)
+    for (int e = 0; t < ends[r]; ++t, ++e) {
+      const size_t at = ((size_t)(e / 4) * nq + r) * 4 + e % 4;
+      E.box[at] = ents[t].sel * A + (ents[t].i - T.imin) + (ents[t].j - T.jmin) * bw;
+      E.w[at] = ents[t].w;
+    }
+  return (double)ents.size() < kMinTileReuse * A * T.nsel ? -nq : nq;
 }
 
-// Levels a staged CSR or transpose tile must hold at once: a full lane
-// group (fewer only when the chunk or the block has fewer).
-int tile_need(int chunk, int L) { return std::min(kTileLevels, std::min(chunk, L)); }
-
-// Staged CSR rows of component ci of sub-matrix s (levels in chunks of
-// `chunk`): tiles of kTileCells rows (16 or 8 when the boxes of 32 rows are
-// too large) whose entries all lie in one 2-D block, in at most two of its
-// slots, inside a box of which a lane group of levels fits a warp's staging
-// area.  Writes the entries' csr_box words.  Returns false (the component
-// keeps the per-lane path) when some tile does not qualify.
-bool emit_csr_tiles(bc_plan* P, const Sub& s, int ci, const Item& proto, int chunk,
-                    std::vector<Item>& out) {
+// Staged CSR rows of component ci of sub-matrix s.  Returns false (the
+// component keeps the per-lane path) when some row does not qualify.
+bool emit_csr_tiles(bc_plan* P, const Sub& s, int ci, const Item& proto, std::vector<Item>& out) {
   const int L = P->blocks[s.block].nlevels;
   const int w = s.ell_w;
-  const int need = tile_need(chunk, L);
+  // rows of one entry read nothing twice: they take the shorter chain
+  const auto nnz0 = P->csr_nnz.begin() + (s.table + ci * s.vol);
+  if (*std::max_element(nnz0, nnz0 + s.vol) <= 1) return false;
   std::vector<Item> tiles;
-  std::vector<std::pair<size_t, int32_t>> boxes;
-  for (int rows = kTileCells; rows >= 8; rows /= 2) {
-    tiles.clear();
-    boxes.clear();
-    bool smaller = false;
-    for (int q0 = 0; q0 < s.vol && !smaller; q0 += rows) {
-      const int nq = std::min(rows, s.vol - q0);
-      TileBox T;
-      for (int q = 0; q < nq; ++q) {
-        const size_t row = (size_t)(s.table + ci * s.vol + q0 + q);
-        const size_t e0 = (size_t)s.ell_base + ((size_t)ci * s.vol + q0 + q) * w;
-        for (int k = 0; k < P->csr_nnz[row]; ++k)
-          if (!T.add(P, e0 + k, P->csr_slot[e0 + k], P->csr_off[e0 + k])) return false;
-      }
-      const int r = finish_tile(P, T, q0, nq, proto, chunk, L, need, kStageBytesCsr, tiles, boxes);
-      if (r < 0) return false;
-      smaller = r == 0;
+  TileEntries all, E;
+  auto entries = [&](int q, auto f) {
+    const size_t e0 = (size_t)s.ell_base + ((size_t)ci * s.vol + q) * w;
+    for (int k = 0; k < P->csr_nnz[(size_t)(s.table + ci * s.vol + q)]; ++k)
+      f(P->csr_slot[e0 + k], P->csr_off[e0 + k], P->csr_val[e0 + k]);
+  };
+  for (int q0 = 0; q0 < s.vol;) {
+    TileBox T;
+    const int nq = grow_tile(P, q0, s.vol, L, kPlaneCsr, entries, T, E);
+    if (nq <= 0) return false;
+    Item it = proto;
+    it.src_org = (int32_t)(P->tile_box.size() + all.box.size());
+    // rows of blocks of 8 entries read whole blocks: pad the last one
+    if (it.p % 8 == 0 && (E.box.size() / 4 / nq) % 2) {
+      E.box.resize(E.box.size() + 4 * nq, 0);
+      E.w.resize(E.w.size() + 4 * nq, 0.0);
     }
-    if (smaller) continue;
-    for (const auto& b : boxes) P->csr_box[b.first] = b.second;
-    out.insert(out.end(), tiles.begin(), tiles.end());
-    return true;
+    push_tile(P, T, q0, nq, it, L, tiles);
+    all.box.insert(all.box.end(), E.box.begin(), E.box.end());
+    all.w.insert(all.w.end(), E.w.begin(), E.w.end());
+    q0 += nq;
   }
-  return false;
+  if (P->tile_box.size() + all.box.size() > INT32_MAX) return false;
+  P->tile_box.insert(P->tile_box.end(), all.box.begin(), all.box.end());
+  P->tile_w.insert(P->tile_w.end(), all.w.begin(), all.w.end());
+  out.insert(out.end(), tiles.begin(), tiles.end());
+  return true;
 }
 
-// Staged transpose rows [r0, r0 + nrows) (one data slot, levels in chunks
-// of `chunk`, the chunked unit order): tiles of kTileCells rows (16 or 8
-// when some box of 32 rows is too large); a tile that does not qualify
-// keeps the per-lane gather (one item of its rows per level chunk).
-// Returns false, emitting nothing, when no tile qualifies.
+// Staged transpose rows [r0, r0 + nrows) (one data slot; per-lane rows in
+// chunks of `chunk` levels).  Rows that cannot be staged keep the per-lane
+// gather (items of up to 32 rows and one level chunk).  Returns false,
+// emitting nothing, when no row can.
 bool emit_adj_tiles(bc_plan* P, int r0, int nrows, const Item& proto, int chunk, int L,
                     std::vector<Item>& out) {
-  const int need = tile_need(chunk, L);
   std::vector<Item> items;
-  std::vector<std::pair<size_t, int32_t>> boxes;
-  int staged = 0;
-  for (int rows = kTileCells; rows >= 8; rows /= 2) {
-    items.clear();
-    boxes.clear();
-    staged = 0;
-    bool smaller = false;
-    for (int q0 = 0; q0 < nrows && !smaller; q0 += rows) {
-      const int nq = std::min(rows, nrows - q0);
-      TileBox T;
-      bool ok = true;
-      for (int q = 0; q < nq && ok; ++q) {
-        const size_t r = (size_t)(r0 + q0 + q);
-        for (int64_t e = P->adj_ptr[r]; e < P->adj_ptr[r + 1] && ok; ++e)
-          ok = T.add(P, (size_t)e, P->aent_slot[(size_t)e], P->aent_off[(size_t)e]);
-      }
-      const int res =
-          ok ? finish_tile(P, T, q0, nq, proto, chunk, L, need, kStageBytesRows, items, boxes) : -1;
-      if (res > 0) {
-        ++staged;
-        continue;
-      }
-      if (res == 0 && rows > 8) {
-        smaller = true;
-        continue;
-      }
+  TileEntries all, E;
+  auto entries = [&](int q, auto f) {
+    const size_t r = (size_t)(r0 + q);
+    for (int64_t e = P->adj_ptr[r]; e < P->adj_ptr[r + 1]; ++e)
+      f(P->aent_slot[(size_t)e], P->aent_off[(size_t)e], P->aent_w[(size_t)e]);
+  };
+  bool staged = false;
+  int plain0 = 0;  // first row of the pending unstaged ones
+  auto flush = [&](int end) {
+    for (int q0 = plain0; q0 < end; q0 += kTileCells)
       for (int c = 0; c * chunk < L; ++c) {
         Item it = proto;
         it.mode = chunk;
         it.u0 = q0 + c * nrows;
-        it.nunits = nq;
+        it.nunits = std::min(kTileCells, end - q0);
         items.push_back(it);
       }
+  };
+  for (int q0 = 0; q0 < nrows;) {
+    TileBox T;
+    const int nq = grow_tile(P, q0, nrows, L, kPlaneAdj, entries, T, E);
+    if (nq <= 0) {
+      q0 += std::max(1, -nq);
+      continue;
     }
-    if (!smaller) break;
+    flush(q0);
+    Item it = proto;
+    it.src_org = (int32_t)(P->tile_box.size() + all.box.size());
+    push_tile(P, T, q0, nq, it, L, items);
+    all.box.insert(all.box.end(), E.box.begin(), E.box.end());
+    all.w.insert(all.w.end(), E.w.begin(), E.w.end());
+    staged = true;
+    q0 += nq;
+    plain0 = q0;
   }
-  if (!staged) return false;
-  for (const auto& b : boxes) P->adj_box[b.first] = b.second;
+  flush(nrows);
+  if (!staged || P->tile_box.size() + all.box.size() > INT32_MAX) return false;
+  P->tile_box.insert(P->tile_box.end(), all.box.begin(), all.box.end());
+  P->tile_w.insert(P->tile_w.end(), all.w.begin(), all.w.end());
   out.insert(out.end(), items.begin(), items.end());
   return true;
 }
 
 void build_items(bc_plan* P) {
   P->runs.clear();
-  P->adj_box.assign(P->aent_off.size(), 0);
   P->itp_box.assign(P->itp_idx.size(), 0);
-  P->csr_box.assign(P->csr_off.size(), 0);
+  P->tile_box.clear();
+  P->tile_w.clear();
   // units per warp item: single-level values (flat) or 8-level chunks
   const int upl = std::max(1, std::min(P->opts.units_per_lane, 64));
   // A small plan still gets enough items to keep every SM busy: the value
@@ -1296,7 +1333,10 @@ void build_items(bc_plan* P) {
   }
   auto table_emit = [&](std::vector<Item>& out, const Item& it, const bc_block& B, int vol) {
     const bool interp = it.kind == IK_INTERP || it.kind == IK_INTERP_PAIR;
-    const int mode = table_mode(B, P->opts.unit_order, level_chunk(P, interp));
+    const int mode = table_mode(B, P->opts.unit_order,
+                                it.kind == IK_CSR ? level_chunk(P, FAM_CSR)
+                                : interp          ? level_chunk(P, FAM_INTERP)
+                                                  : level_chunk(P, FAM_ADJ));
     emit_units(out, it, vol, B.nlevels, mode, mode < 2 ? per_table_flat_item : per_table_item);
   };
   std::vector<std::pair<int, std::vector<Item>>> per_sub(P->subs.size());
@@ -1340,9 +1380,9 @@ void build_items(bc_plan* P) {
           }
           // levels far apart in memory: stage the nodes of each tile in
           // shared memory when the tiles' boxes are small
-          const int mode = table_mode(B, P->opts.unit_order, level_chunk(P, true));
+          const int mode = table_mode(B, P->opts.unit_order, level_chunk(P, FAM_INTERP));
           if (mode < 2 || P->opts.unstaged_rows ||
-              !emit_tiles(P, s, it, mode, it.kind == IK_INTERP_PAIR ? 2 : 1, out))
+              !emit_tiles(P, s, it, out))
             table_emit(out, it, B, s.vol);
           break;
         }
@@ -1357,9 +1397,9 @@ void build_items(bc_plan* P) {
             it.src_ls = (int32_t)(S.nlevels > 1 ? S.level_stride : 0);
           }
           // levels far apart in memory: stage each tile's column box
-          const int mode = table_mode(B, P->opts.unit_order, level_chunk(P, false));
+          const int mode = table_mode(B, P->opts.unit_order, level_chunk(P, FAM_CSR));
           if (mode < 2 || P->opts.unstaged_rows ||
-              !emit_csr_tiles(P, s, (int)ci, it, mode, out))
+              !emit_csr_tiles(P, s, (int)ci, it, out))
             table_emit(out, it, B, s.vol);
           break;
         }
@@ -1426,7 +1466,11 @@ void build_items(bc_plan* P) {
         case IK_MAP: return 2 * vals;
         case IK_INTERP: return vals * (2 + it.p / 2);
         case IK_INTERP_PAIR: return vals * 2 * (2 + it.p / 2);
-        default: return vals * (1 + it.p);
+        default:
+          // rows that read several slots first: theirs is the longest chain
+          // of dependent loads (entry, slot pointer, level stride, value)
+          if (it.mode != MODE_TILE && it.src_slot < 0) return INT64_MAX;
+          return vals * (1 + it.p);
       }
     };
     std::vector<Item> all;
@@ -1499,7 +1543,7 @@ void build_items(bc_plan* P) {
       it.src_ls = (int32_t)(G.nlevels > 1 ? G.level_stride : 0);
     }
     // levels far apart in memory: stage each tile's box of ghost cotangents
-    const int mode = table_mode(B0, P->opts.unit_order, level_chunk(P, false));
+    const int mode = table_mode(B0, P->opts.unit_order, level_chunk(P, FAM_ADJ));
     if (mode < 2 || P->opts.unstaged_rows ||
         !emit_adj_tiles(P, r0, r1 - r0, it, mode, B0.nlevels, P->adj_items))
       table_emit(P->adj_items, it, B0, r1 - r0);
@@ -1507,10 +1551,11 @@ void build_items(bc_plan* P) {
   }
   P->adj_items.insert(P->adj_items.begin(), P->adj_add.begin(), P->adj_add.end());
   // the shared-memory stage each launch requests per warp
-  auto stage_of = [](const std::vector<Item>& v) {
+  auto stage_of = [P](const std::vector<Item>& v) {
     int b = 0;
     for (const Item& it : v)
-      if (it.mode == MODE_TILE) b = std::max(b, it.kind == IK_CSR ? kStageBytesCsr : kStageBytesRows);
+      if (it.mode == MODE_TILE)
+        b = std::max(b, stage_bytes(it.kind == IK_CSR, it.kind != IK_INTERP, P->esize));
     return b;
   };
   for (int f = 0; f < kFamilies; ++f) P->staged[f] = stage_of(P->fam_items[f]);
@@ -1842,14 +1887,17 @@ bc_status upload_work(bc_plan* P) {
   const size_t o_z = L.take(P->adj_zero.size() * sizeof(Item));
   const size_t o_all = L.take(P->all_items.size() * sizeof(Item));
   const size_t o_box = L.take(P->itp_box.size() * 4);
-  const size_t o_cbox = L.take(P->csr_box.size() * 4);
-  const size_t o_abox = L.take(P->adj_box.size() * 4);
+  const size_t o_tbox = L.take(P->tile_box.size() * 4);
+  const size_t o_tw = L.take(P->tile_w.size() * P->esize);
   std::vector<char> host(L.off + 256, 0);
   put_raw(host, o_i, P->items);
   put_raw(host, o_all, P->all_items);
   put_raw(host, o_box, P->itp_box);
-  put_raw(host, o_cbox, P->csr_box);
-  put_raw(host, o_abox, P->adj_box);
+  put_raw(host, o_tbox, P->tile_box);
+  if (P->dtype == BC_F64)
+    put_dtype<double>(host, o_tw, P->tile_w);
+  else
+    put_dtype<float>(host, o_tw, P->tile_w);
   for (int f = 0; f < kFamilies; ++f) put_raw(host, o_f[f], P->fam_items[f]);
   put_raw(host, o_r, P->runs);
   put_raw(host, o_a, P->adj_items);
@@ -1870,8 +1918,8 @@ bc_status upload_work(bc_plan* P) {
   P->d_adj_zero = reinterpret_cast<Item*>(b + o_z);
   P->d_all = reinterpret_cast<Item*>(b + o_all);
   P->ctx.itp_box = reinterpret_cast<const int32_t*>(b + o_box);
-  P->ctx.csr_box = reinterpret_cast<const int32_t*>(b + o_cbox);
-  P->ctx.adj_box = reinterpret_cast<const int32_t*>(b + o_abox);
+  P->ctx.tile_box = reinterpret_cast<const int32_t*>(b + o_tbox);
+  P->ctx.tile_w = b + o_tw;
   return BC_OK;
 }
 
@@ -2718,6 +2766,11 @@ struct WorkCheck {
   }
 };
 
+// place of entry k of row q of a staged CSR or transpose tile
+size_t tile_entry(const Item& it, int q, int k) {
+  return (size_t)it.src_org + ((size_t)(k / 4) * it.nunits + (size_t)(q - it.u0)) * 4 + k % 4;
+}
+
 int64_t check_forward_list(WorkCheck& W, const std::vector<Item>& items, bool values = true) {
   const bc_plan* P = W.P;
   const ExplicitRows& R = P->rows;
@@ -2783,12 +2836,15 @@ int64_t check_forward_list(WorkCheck& W, const std::vector<Item>& items, bool va
         const int nnz = P->csr_nnz[row];
         std::vector<std::pair<int64_t, double>> a, b;
         for (int k = 0; k < nnz; ++k) {
-          const size_t e = (size_t)it.src_org + (size_t)q * (size_t)it.p + (size_t)k;
+          const size_t e = it.mode == MODE_TILE ? 0 : (size_t)it.src_org + (size_t)q * (size_t)it.p + (size_t)k;
           int slot = it.src_slot >= 0 ? it.src_slot : P->csr_slot[e];
           int64_t off = P->csr_off[e];
+          double val = P->csr_val[e];
           if (it.mode == MODE_TILE) {
             // a staged row reads its column from the tile's box
-            const int32_t bx = P->csr_box[e], A = it.bw * it.bh;
+            const size_t t = tile_entry(it, q, k);
+            const int32_t bx = P->tile_box[t], A = it.bw * it.bh;
+            val = P->tile_w[t];
             const int idx = bx % A;
             slot = bx / A ? it.bsrc2 : it.bsrc;
             off = it.borg + (int64_t)(idx % it.bw) * it.bs0 + (int64_t)(idx / it.bw) * it.bs1;
@@ -2796,7 +2852,7 @@ int64_t check_forward_list(WorkCheck& W, const std::vector<Item>& items, bool va
               W.problem("a staged CSR entry lies outside its box", it.dst_slot, E);
           }
           const int64_t ls = it.src_slot >= 0 ? it.src_ls : W.ls_of_slot(slot);
-          a.push_back({col_key(slot, off + l * ls), P->csr_val[e]});
+          a.push_back({col_key(slot, off + l * ls), val});
         }
         for (int64_t e = R.ptr[w->r]; e < R.ptr[w->r + 1]; ++e)
           b.push_back({col_key(R.cslot[e], R.coff[e] + w->l * W.ls_of_slot(R.cslot[e])), R.val[e]});
@@ -2896,9 +2952,12 @@ int64_t check_adjoint_lists(WorkCheck& W, const std::vector<Item>& adj_items) {
       for (int64_t e = P->adj_ptr[tr]; e < P->adj_ptr[tr + 1]; ++e) {
         int gs = P->aent_slot[(size_t)e];
         int64_t go = P->aent_off[(size_t)e];
+        double val = P->aent_w[(size_t)e];
         if (it.mode == MODE_TILE) {
           // a staged row reads its ghost value from the tile's box
-          const int32_t bx = P->adj_box[(size_t)e], A = it.bw * it.bh;
+          const size_t t = tile_entry(it, q, (int)(e - P->adj_ptr[tr]));
+          const int32_t bx = P->tile_box[t], A = it.bw * it.bh;
+          val = P->tile_w[t];
           const int idx = bx % A;
           gs = bx / A ? it.bsrc2 : it.bsrc;
           go = it.borg + (int64_t)(idx % it.bw) * it.bs0 + (int64_t)(idx / it.bw) * it.bs1;
@@ -2909,7 +2968,7 @@ int64_t check_adjoint_lists(WorkCheck& W, const std::vector<Item>& adj_items) {
         if (order < prev)
           W.problem("transpose entries out of ghost order", it.dst_slot, P->arow_off[tr]);
         prev = order;
-        got[d].push_back({col_key(gs, go + l * W.ls_of_slot(gs)), P->aent_w[(size_t)e]});
+        got[d].push_back({col_key(gs, go + l * W.ls_of_slot(gs)), val});
       }
     });
   }
