@@ -148,6 +148,9 @@ struct Ctx {
   // values that read them
   const int32_t* arow_slot;
   const int32_t* arow_off;
+  // a row and its first two entries: {data offset, entries, first entry, ghost
+  // offset 0}, {ghost offset 1, weights 0 and 1 (FP32)}, FP64 also {weights}
+  const int4* arow_rec;
   const int64_t* adj_ptr;
   const int32_t* aent_slot;
   const int32_t* aent_off;

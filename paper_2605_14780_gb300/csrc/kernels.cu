@@ -1148,16 +1148,91 @@ __device__ void adj_chunk(const Item& item, const Ptrs& P, const Ctx& c, int lan
   }
 }
 
+// Flat transpose rows.  Bound by the chain of dependent loads (row, entries,
+// ghost values; about 1 us a value at the 28 warps an SM holds) and issue, so
+// rows whose entries read one slot (P.s) come as records that hold the row
+// and its first two entries (Ctx::arow_rec; most rows of user CSR edges have
+// no more) and a lane takes U values through the two steps side by side.  512
+// blocks, levels innermost, FP32: the adjoint 97 us with the row pointers and
+// entries in their own arrays, 103 with records and U = 1, 84 with 2, 80 with
+// 3, 86 with 4 (spills); FP64 gains nothing past 1.
 template <typename T>
-__device__ void adj_flat(const Item& it, const Ptrs& P, const Ctx& c, int lane) {
+struct AdjRec {  // int4s of one record
+  static constexpr int n = sizeof(T) == 4 ? 2 : 3;
+};
+
+template <typename T>
+__device__ void adj_flat(const Item& item, const Ptrs& P, const Ctx& c, int lane) {
   constexpr int E = kAdjBatch;
+  const Item it = item;
   const int end = it.u0 + it.nunits;
   const T* wv = static_cast<const T*>(c.aent_w);
+  const T* yb = static_cast<const T*>(P.s);
+  T* xd = static_cast<T*>(P.d);
+  if (yb) {
+    constexpr int U = sizeof(T) == 4 ? 3 : 1;
+    const int4* rec = c.arow_rec + (size_t)it.table * AdjRec<T>::n;
+    for (int f0 = it.u0 + lane; f0 < end; f0 += 32 * U) {
+      // straight through, without branches, so that the U values' loads of
+      // each step issue together: values past the end repeat the last one, a
+      // single entry stands for both
+      int4 ra[U], rb[U], rc[U];
+      int lv[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        int q;
+        flat_of(min(f0 + 32 * u, end - 1), it, q, lv[u]);
+        const int4* rp = rec + q * AdjRec<T>::n;
+        ra[u] = __ldg(rp);
+        rb[u] = __ldg(rp + 1);
+        if constexpr (sizeof(T) == 8) rc[u] = __ldg(rp + 2);
+      }
+      T x[U], y0[U], y1[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const T* yl = yb + lv[u] * it.src_ls;
+        x[u] = xd[ra[u].x + lv[u] * it.dst_ls];
+        y0[u] = yl[ra[u].w];
+        y1[u] = yl[rb[u].x];
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        T w0, w1;
+        if constexpr (sizeof(T) == 4) {
+          w0 = __int_as_float(rb[u].y);
+          w1 = __int_as_float(rb[u].z);
+        } else {
+          w0 = __hiloint2double(rc[u].y, rc[u].x);
+          w1 = __hiloint2double(rc[u].w, rc[u].z);
+        }
+        const int n = ra[u].y;
+        T acc = fma(w0, y0[u], x[u]);
+        acc = n > 1 ? fma(w1, y1[u], acc) : acc;
+        if (n > 2) {
+          const T* yl = yb + lv[u] * it.src_ls;
+          for (int eb = ra[u].z + 2, e1 = ra[u].z + n; eb < e1; eb += E) {
+            T y[E], a[E];
+#pragma unroll
+            for (int e = 0; e < E; ++e)
+              if (eb + e < e1) {
+                y[e] = yl[__ldg(c.aent_off + eb + e)];
+                a[e] = ldg(wv + eb + e);
+              }
+#pragma unroll
+            for (int e = 0; e < E; ++e)
+              if (eb + e < e1) acc = fma(a[e], y[e], acc);
+          }
+        }
+        if (f0 + 32 * u < end) xd[ra[u].x + lv[u] * it.dst_ls] = acc;
+      }
+    }
+    return;
+  }
   for (int f = it.u0 + lane; f < end; f += 32) {
     int q, l;
     flat_of(f, it, q, l);
     const int r = it.table + q;
-    T* xb = static_cast<T*>(P.d) + (__ldg(c.arow_off + r) + l * it.dst_ls);
+    T* xb = xd + (__ldg(c.arow_off + r) + l * it.dst_ls);
     const int e0 = (int)__ldg(c.adj_ptr + r), e1 = (int)__ldg(c.adj_ptr + r + 1);
     T acc = *xb;
     for (int eb = e0; eb < e1; eb += E) {
@@ -1165,15 +1240,9 @@ __device__ void adj_flat(const Item& it, const Ptrs& P, const Ctx& c, int lane) 
 #pragma unroll
       for (int e = 0; e < E; ++e)
         if (eb + e < e1) {
-          const T* yp;
-          if (P.s) {
-            yp = static_cast<const T*>(P.s) + (__ldg(c.aent_off + eb + e) + l * it.src_ls);
-          } else {
-            const int gs = __ldg(c.aent_slot + eb + e);
-            yp = static_cast<const T*>(c.slots[gs]) +
-                 (__ldg(c.aent_off + eb + e) + l * __ldg(c.slot_ls + gs));
-          }
-          y[e] = *yp;
+          const int gs = __ldg(c.aent_slot + eb + e);
+          y[e] = *(static_cast<const T*>(c.slots[gs]) +
+                   (__ldg(c.aent_off + eb + e) + l * __ldg(c.slot_ls + gs)));
           a[e] = ldg(wv + eb + e);
         }
 #pragma unroll

@@ -864,11 +864,12 @@ int table_mode(const bc_block& B, int order, int chunk) {
 
 // levels per unit of the chunked unit order (bc_plan_opts.level_chunk; by
 // default 4 for interpolation rows, whose pair path keeps two components'
-// sums, and 8 for CSR and transpose rows); the persistent launch's kernel
-// holds at most 4
+// sums, and for transpose rows, whose longest chain ends the launch
+// (the 6 x 768^2 adjoint 107 us at 8, 79 us at 4), and 8 for CSR rows); the persistent launch's kernel holds at
+// most 4
 int level_chunk(const bc_plan* P, int fam) {
   int ch = P->opts.level_chunk;
-  if (ch == 0) ch = fam == FAM_INTERP ? 4 : 8;
+  if (ch == 0) ch = fam == FAM_CSR ? 8 : 4;
   const bool all_kinds =
       P->opts.batch_mode == BC_BATCH_PERSISTENT || P->opts.batch_mode == BC_BATCH_SINGLE;
   return all_kinds ? std::min(ch, 4) : ch;
@@ -1304,7 +1305,16 @@ void build_items(bc_plan* P) {
   // table-driven kinds (interpolation, CSR, transpose): one unit per lane, so
   // a warp's dependent table -> data chains run side by side, not in series
   const int per_table_item = 32;
-  const int per_table_flat_item = std::min(32 * 8, small);
+  // Flat items of table-driven kinds take at least 8 values a lane only in
+  // plans of kTableItemsPerSm items an SM: each value is a chain of dependent
+  // loads, so warps side by side beat values in series (6 x 91^2 x 37 levels
+  // FP64, levels innermost, forward and adjoint: 77 us at 16 items an SM, 65
+  // at 48, 56 at 96, 50 at 128, 51 at 256).
+  constexpr int kTableItemsPerSm = 128;
+  const int64_t want_table = (int64_t)std::max(1, P->num_sms) * kTableItemsPerSm;
+  const int per_table_flat_item = (int)std::min<int64_t>(
+      32 * 8,
+      std::max<int64_t>(32, (total_values + want_table - 1) / want_table + 31) / 32 * 32);
   auto structured_emit = [&](std::vector<Item>& out, const Item& it, const bc_block& B, int vol) {
     int mode = structured_mode(B, P->opts.unit_order);
     if (mode == MODE_FLAT_CELL && B.nlevels > 1) {
@@ -1520,15 +1530,24 @@ void build_items(bc_plan* P) {
   // one ghost slot, that slot is resolved once too
   P->adj_items.clear();
   const int nar = (int)P->arow_slot.size();
+  auto one_reader = [P](int r) {
+    const int64_t e0 = P->adj_ptr[r], e1 = P->adj_ptr[r + 1];
+    for (int64_t e = e0 + 1; e < e1; ++e)
+      if (P->aent_slot[e] != P->aent_slot[e0]) return -1;
+    return e0 < e1 ? P->aent_slot[e0] : -1;
+  };
   int r0 = 0;
   while (r0 < nar) {
     const int ds = P->arow_slot[r0];
     const bc_block& B0 = P->blocks[P->slot_block[ds]];
-    int r1 = r0;
-    while (r1 < nar && P->arow_slot[r1] == ds) ++r1;
-    int common = -2;
-    for (int64_t e = P->adj_ptr[r0]; e < P->adj_ptr[r1] && common != -1; ++e)
-      common = common == -2 ? P->aent_slot[e] : (common == P->aent_slot[e] ? common : -1);
+    // consecutive rows of the slot whose entries all read one ghost slot (or
+    // none of them do)
+    int r1 = r0, common = -1;
+    for (; r1 < nar && P->arow_slot[r1] == ds; ++r1) {
+      const int c = one_reader(r1);
+      if (r1 == r0) common = c;
+      else if (c != common) break;
+    }
     Item it{};
     it.kind = IK_ADJ;
     it.vol = make_div((uint32_t)(r1 - r0));
@@ -1550,6 +1569,34 @@ void build_items(bc_plan* P) {
     r0 = r1;
   }
   P->adj_items.insert(P->adj_items.begin(), P->adj_add.begin(), P->adj_add.end());
+  // Longest first, by the steps of a lane's serial chain: the few rows that
+  // stay out of the tiles (data values at the corners of a panel, read by
+  // tens of ghosts) would otherwise start last and end alone (6 x 768^2 x 96 planes: 115 ->
+  // 107 us; 512 blocks, levels innermost: 101 -> 97 us).
+  {
+    auto steps = [&](const Item& it) -> int64_t {
+      if (it.kind == IK_ADD) {
+        int64_t n = 0;
+        for (int r = it.u0; r < it.u0 + it.nunits; ++r) n += P->runs[(size_t)r].z;
+        return n / 256;
+      }
+      const bool flat = it.mode == MODE_FLAT_CELL || it.mode == MODE_FLAT_LEVEL;
+      const int per = flat && it.mode == MODE_FLAT_LEVEL ? (int)it.lev.d : 1;
+      const int vol = (int)it.vol.d;
+      int64_t nnz = 0;
+      for (int u = it.u0 / per; u <= (it.u0 + it.nunits - 1) / per; ++u) {
+        const size_t r = (size_t)(it.table + (it.mode == MODE_TILE ? u : u % vol));
+        nnz = std::max(nnz, P->adj_ptr[r + 1] - P->adj_ptr[r]);
+      }
+      return it.mode == MODE_TILE ? 1 + nnz / 4 : (nnz + 3) / 4 * (flat ? (it.nunits + 31) / 32 : 4);
+    };
+    std::vector<std::pair<int64_t, size_t>> key(P->adj_items.size());
+    for (size_t t = 0; t < key.size(); ++t) key[t] = {-steps(P->adj_items[t]), t};
+    std::stable_sort(key.begin(), key.end());
+    std::vector<Item> sorted(key.size());
+    for (size_t t = 0; t < key.size(); ++t) sorted[t] = P->adj_items[key[t].second];
+    P->adj_items.swap(sorted);
+  }
   // the shared-memory stage each launch requests per warp
   auto stage_of = [P](const std::vector<Item>& v) {
     int b = 0;
@@ -1644,21 +1691,27 @@ void split_unit_copies(bc_plan* P) {
   P->adj_ptr.swap(ptr);
 }
 
-// Within each data slot, the transpose rows read by one ghost slot (the
-// slot of their first entry) are made consecutive, in data-offset order:
-// consecutive rows then gather from one neighbour strip, so tiles of them
-// can stage that strip (and more items find one common ghost slot).  Each
-// data value keeps its one row and its entries' ghost order.
+// Within each data slot, the transpose rows whose entries read one ghost slot
+// are made consecutive by that slot, then those that read several (by the
+// slot of their first entry), in data-offset order: consecutive rows then
+// gather from one neighbour strip, so tiles of them can stage that strip and
+// items find one common ghost slot.  Each data value keeps its one row and
+// its entries' ghost order.
 void group_rows_by_reader(bc_plan* P) {
   const size_t nr = P->arow_slot.size();
   std::vector<size_t> order(nr);
   std::iota(order.begin(), order.end(), size_t(0));
-  auto reader = [&](size_t r) {
-    return P->adj_ptr[r + 1] > P->adj_ptr[r] ? P->aent_slot[(size_t)P->adj_ptr[r]] : -1;
-  };
+  std::vector<int64_t> reader(nr, -1);
+  for (size_t r = 0; r < nr; ++r) {
+    const int64_t e0 = P->adj_ptr[r], e1 = P->adj_ptr[r + 1];
+    if (e0 == e1) continue;
+    bool one = true;
+    for (int64_t e = e0 + 1; e < e1; ++e) one = one && P->aent_slot[e] == P->aent_slot[e0];
+    reader[r] = P->aent_slot[e0] + (one ? 0 : (int64_t)P->nslots);
+  }
   std::stable_sort(order.begin(), order.end(), [&](size_t a, size_t b) {
     if (P->arow_slot[a] != P->arow_slot[b]) return P->arow_slot[a] < P->arow_slot[b];
-    return reader(a) < reader(b);
+    return reader[a] < reader[b];
   });
   std::vector<int32_t> rs(nr), ro(nr), es, eo;
   std::vector<int64_t> ptr{0};
@@ -1753,6 +1806,26 @@ void put_raw(std::vector<char>& host, size_t off, const std::vector<V>& v) {
   if (!v.empty()) std::memcpy(host.data() + off, v.data(), v.size() * sizeof(V));
 }
 
+// Ctx::arow_rec of every transpose row.
+std::vector<int4> adjoint_records(const bc_plan* P) {
+  const size_t n = P->arow_off.size(), per = P->dtype == BC_F64 ? 3 : 2;
+  std::vector<int4> rec(n * per, make_int4(0, 0, 0, 0));
+  for (size_t r = 0; r < n; ++r) {
+    const size_t e0 = (size_t)P->adj_ptr[r], m = (size_t)(P->adj_ptr[r + 1] - P->adj_ptr[r]);
+    int4* at = &rec[r * per];
+    at[0] = make_int4(P->arow_off[r], (int)m, (int)e0, m > 0 ? P->aent_off[e0] : 0);
+    at[1].x = m > 1 ? P->aent_off[e0 + 1] : at[0].w;
+    const double w[2] = {m > 0 ? P->aent_w[e0] : 0.0, m > 1 ? P->aent_w[e0 + 1] : 0.0};
+    if (P->dtype == BC_F64) {
+      std::memcpy(&at[2], w, sizeof(w));
+    } else {
+      const float f[2] = {(float)w[0], (float)w[1]};
+      std::memcpy(&at[1].y, f, sizeof(f));
+    }
+  }
+  return rec;
+}
+
 bc_status upload_tables(bc_plan* P) {
   const size_t S = P->esize;
   Layout L;
@@ -1770,6 +1843,8 @@ bc_status upload_tables(bc_plan* P) {
   const size_t o_k = L.take(P->const_val.size() * S);
   const size_t o_as = L.take(P->arow_slot.size() * 4);
   const size_t o_ao = L.take(P->arow_off.size() * 4);
+  const std::vector<int4> rec = adjoint_records(P);
+  const size_t o_ar = L.take(rec.size() * sizeof(int4));
   const size_t o_ap = L.take(P->adj_ptr.size() * 8);
   const size_t o_es = L.take(P->aent_slot.size() * 4);
   const size_t o_eo = L.take(P->aent_off.size() * 4);
@@ -1801,6 +1876,7 @@ bc_status upload_tables(bc_plan* P) {
   put_raw(host, o_co, P->csr_off);
   put_raw(host, o_as, P->arow_slot);
   put_raw(host, o_ao, P->arow_off);
+  put_raw(host, o_ar, rec);
   put_raw(host, o_ap, P->adj_ptr);
   put_raw(host, o_es, P->aent_slot);
   put_raw(host, o_eo, P->aent_off);
@@ -1847,6 +1923,7 @@ bc_status upload_tables(bc_plan* P) {
   c.const_val = b + o_k;
   c.arow_slot = reinterpret_cast<const int32_t*>(b + o_as);
   c.arow_off = reinterpret_cast<const int32_t*>(b + o_ao);
+  c.arow_rec = reinterpret_cast<const int4*>(b + o_ar);
   c.adj_ptr = reinterpret_cast<const int64_t*>(b + o_ap);
   c.aent_slot = reinterpret_cast<const int32_t*>(b + o_es);
   c.aent_off = reinterpret_cast<const int32_t*>(b + o_eo);
