@@ -75,10 +75,16 @@ constexpr int kTileCells = 32;
 constexpr int kTileLevels = 4;
 constexpr int stage_levels(int esize) { return esize == 8 ? kTileLevels : 2 * kTileLevels; }
 constexpr int kPlaneInterp = 64, kPlaneCsr = 256, kPlaneAdj = 128;
+// CSR tiles hold one lane group of levels: 4 KB a warp in FP32, so that the
+// 32 warps their registers allow fit an SM (8 levels, 8 KB, 22 warps seen:
+// the 4 x 4 reconstruction rows of 6 x 384^2 65 us against 48; planes of 320
+// elements 48, of 512 66).  Interpolation and transpose tiles hold two (one:
+// 6 x 384^2 fill 24.6 us against 22.8, 6 x 768^2 adjoint 84 against 80).
+constexpr int kCsrStageLevels = kTileLevels;
 // shared memory of one warp's stage
 constexpr int stage_bytes(bool csr, bool pair_or_adj, int esize) {
-  return stage_levels(esize) * esize *
-         (csr ? kPlaneCsr : (pair_or_adj ? kPlaneAdj : kPlaneInterp));
+  return esize * (csr ? kCsrStageLevels * kPlaneCsr
+                      : stage_levels(esize) * (pair_or_adj ? kPlaneAdj : kPlaneInterp));
 }
 static_assert(kPlaneAdj == 2 * kPlaneInterp, "pairs and transpose tiles stage the same bytes");
 

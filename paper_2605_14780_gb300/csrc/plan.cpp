@@ -1023,8 +1023,8 @@ struct TileBox {
 
 // levels of a staged item: equal parts of the block's, at most what the
 // stage holds (fewer with bc_plan_opts.level_chunk)
-int tile_levels(const bc_plan* P, int L) {
-  const int held = stage_levels(P->esize);
+int tile_levels(const bc_plan* P, int L, bool csr) {
+  const int held = csr ? kCsrStageLevels : stage_levels(P->esize);
   const int most = P->opts.level_chunk ? std::min(P->opts.level_chunk, held) : held;
   const int parts = (L + most - 1) / most;
   return (L + parts - 1) / parts;
@@ -1035,7 +1035,7 @@ int tile_levels(const bc_plan* P, int L) {
 void push_tile(const bc_plan* P, const TileBox& T, int q0, int nq, const Item& proto, int L,
                std::vector<Item>& out) {
   const bc_block& S = P->blocks[T.blk];
-  const int nl = tile_levels(P, L);
+  const int nl = tile_levels(P, L, proto.kind == IK_CSR);
   for (int l0 = 0; l0 < L; l0 += nl) {
     Item it = proto;
     it.mode = MODE_TILE;
@@ -1176,7 +1176,7 @@ int grow_tile(const bc_plan* P, int q, int q1, int L, int plane, F entries, Tile
     }
     return full;
   };
-  if (fill(kTileCells) && ends.size() > 16 && tile_levels(P, L) > kTileLevels) fill(16);
+  if (fill(kTileCells) && ends.size() > 16 && tile_levels(P, L, plane == kPlaneCsr) > kTileLevels) fill(16);
   const int nq = (int)ends.size();
   if (nq == 0 || T.blk < 0) return 0;
   const bc_block& S = P->blocks[T.blk];
