@@ -275,17 +275,20 @@ typedef struct bc_plan_opts {
                               over 4096 entries, or cubed-sphere rows
                               generated on the GPU in the same plan,
                               BC_ERR_UNSUPPORTED                             */
-  int32_t batch_mode;      /* how BC_FORM_BATCHED runs: 0 default
-                              (BC_BATCH_FAMILIES), BC_BATCH_PERSISTENT or
-                              BC_BATCH_FAMILIES; bc_plan_autotune times both */
+  int32_t batch_mode;      /* how BC_FORM_BATCHED runs: a bc_batch_mode, or
+                              0, the default: BC_BATCH_FAMILIES, but
+                              BC_BATCH_SINGLE for plans of several kernel
+                              families with at most 2^21 ghost values;
+                              bc_plan_autotune times them                    */
   int32_t scalar_runs;     /* 1: contiguous runs move one 4- or 8-byte value
                               per lane and load; 0 (default): 16-byte vectors,
                               whatever the runs' alignment                   */
   int32_t level_chunk;     /* levels one lane carries through a table row
                               when levels are far apart in memory
                               (interpolation, CSR and transpose rows): 0
-                              default (4 for interpolation rows, 8 for CSR
-                              and transpose rows), or 1, 2, 4, 8 for all;
+                              default (4 for interpolation and transpose
+                              rows, 8 for CSR rows; staged tiles as many as
+                              they hold), or 1, 2, 4, 8 for all;
                               the launches of every kind in one kernel
                               (BC_BATCH_PERSISTENT, BC_BATCH_SINGLE) take
                               at most 4                                     */
@@ -293,8 +296,7 @@ typedef struct bc_plan_opts {
                               read their columns from global memory lane by
                               lane; 0 (default): with levels far apart in
                               memory, a warp first copies the small box of
-                              cells a tile of 32 rows (16 or 8 when a group
-                              of 4 levels of the box would not fit) reads,
+                              cells a tile of up to 32 rows reads,
                               in at most two slots of one block, into
                               shared memory                                 */
   int32_t stencil_fusion;  /* 1: also build the tables bc_apply_stencil

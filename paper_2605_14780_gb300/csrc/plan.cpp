@@ -2321,6 +2321,9 @@ struct Fnv {
   void val(const V& v) { bytes(&v, sizeof(V)); }
 };
 
+// ghost values up to which a plan of several families runs in one launch
+constexpr int64_t kSingleLaunchValues = 1 << 21;
+
 uint64_t plan_hash(const bc_plan* P) {
   Fnv f;
   f.val(P->dtype);
@@ -2491,6 +2494,21 @@ bc_status plan_create_impl(const bc_grid* grid, const bc_submatrix* subs, int32_
       }
     }
     P->rows = std::move(all);
+  }
+  if (!opts || opts->batch_mode == 0) {
+    // Default mode: small plans of several families take one launch.  Fork
+    // and join cost about 3.5 us a call (a 6 x 32^2 scalar: 10.5 us with two
+    // families, 6.8 us in one launch), against register limits shared by all
+    // kinds: spheres and blocks of 26 k to 1.6 M values gain 3-4.5 us each,
+    // 2.7 M FP32 values are even (22.8 us), 11.7 M lose 2 us of 43.
+    int64_t values = 0;
+    bool has[kFamilies] = {false, false, false, false};
+    for (const Sub& s : P->subs) {
+      values += (int64_t)s.comps.size() * s.vol * P->blocks[s.block].nlevels;
+      has[family_of_kind(s.kind)] = true;
+    }
+    if (has[FAM_STRUCT] + has[FAM_INTERP] + has[FAM_CSR] > 1 && values <= kSingleLaunchValues)
+      P->opts.batch_mode = BC_BATCH_SINGLE;
   }
   if (!P->opts.no_adjoint) build_transpose(P);
   P->hash = plan_hash(P);
