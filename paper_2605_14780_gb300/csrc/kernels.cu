@@ -39,21 +39,36 @@ __device__ __forceinline__ uint32_t fdiv(uint32_t n, const FastDiv& f) {
   return (__umulhi(n, f.m) + n) >> f.s;
 }
 
-// flat unit f -> (cell q, level l)
+// MODE_FLAT_CELL unit f -> (cell q, level l)
 __device__ __forceinline__ void flat_of(int f, const Item& it, int& q, int& l) {
-  if (it.mode == MODE_FLAT_LEVEL) {
-    q = (int)fdiv((uint32_t)f, it.lev);
-    l = f - q * (int)it.lev.d;
-  } else {
-    l = (int)fdiv((uint32_t)f, it.vol);
-    q = f - l * (int)it.vol.d;
-  }
+  l = (int)fdiv((uint32_t)f, it.vol);
+  q = f - l * (int)it.vol.d;
 }
 
 // chunk unit u -> cell q of the box and level chunk c (u = q + vol * c)
 __device__ __forceinline__ void unit_of(int u, const Item& it, int& q, int& c) {
   c = (int)fdiv((uint32_t)u, it.vol);
   q = u - c * (int)it.vol.d;
+}
+
+// MODE_SPLIT: the row of unit u and its kLevelSplit levels (a level past the
+// last one repeats it; n: those that count)
+struct Split {
+  int q, n, l[kLevelSplit];
+};
+__device__ __forceinline__ Split split_of(int u, const Item& it) {
+  Split s;
+  const int part = (int)it.bwid.d, L = (int)it.lev.d;
+  s.q = (int)fdiv((uint32_t)u, it.bwid);
+  const int l0 = u - s.q * part;
+  s.n = 0;
+#pragma unroll
+  for (int k = 0; k < kLevelSplit; ++k) {
+    const int l = l0 + k * part;
+    s.l[k] = min(l, L - 1);
+    s.n += l < L;
+  }
+  return s;
 }
 
 // element offset (level 0) of cell q of the item's box, from the cell table
@@ -773,9 +788,8 @@ __device__ void rows_tile(const Item& item, const Ptrs& P, const Ctx& c, int lan
   __syncwarp();  // every lane is done with the stage before the next item
 }
 
-// Flat interpolation: each lane keeps U values (cell, level) in flight; with
-// level-fastest order the lanes of a warp share a cell, so its table row is
-// one broadcast load and the node loads of the warp are contiguous.
+// Flat interpolation: each lane keeps U values (cell, level) in flight, cells
+// fastest.
 template <typename T, bool PAIR>
 __device__ void interp_flat(const Item& item, const Ptrs& P, const Ctx& c, int lane) {
   const Item it = item;
@@ -840,24 +854,75 @@ __device__ void interp_flat(const Item& item, const Ptrs& P, const Ctx& c, int l
   }
 }
 
+// Interpolation with contiguous levels (MODE_SPLIT).  Table look-ups and
+// addresses cost as much as the sums, so a lane takes kLevelSplit values of a
+// row, the lanes of a warp consecutive levels: 6 x 91^2 x 37 levels FP64,
+// forward and adjoint, 49.5 -> 47.1 us.
+template <typename T, bool PAIR>
+__device__ void interp_split(const Item& item, const Ptrs& P, const Ctx& c, int lane) {
+  using B = typename BitsOf<T>::type;
+  constexpr int K = kLevelSplit;
+  const Item it = item;
+  const int end = it.u0 + it.nunits;
+  const int p = it.p, dls = it.dst_ls;
+  const int cu = it.comp & 0xffff, cv = it.comp >> 16;
+  for (int u = it.u0 + lane; u < end; u += 32) {
+    const Split t = split_of(u, it);
+    const int row = it.table + t.q;
+    const int4 ix = __ldg(c.itp_idx + row);
+    const int dof = dst_cell(it, c, t.q);
+    const int su = ix.x + cu, sv = ix.x + cv;
+    const int uls = __ldg(c.slot_ls + su), vls = PAIR ? __ldg(c.slot_ls + sv) : 0;
+    const T* xu = static_cast<const T*>(c.slots[su]) + ix.y;
+    const T* xv = PAIR ? static_cast<const T*>(c.slots[sv]) + ix.y : nullptr;
+    B* du = static_cast<B*>(P.d) + dof;
+    B* dv = PAIR ? static_cast<B*>(P.d2) + dof : nullptr;
+    const bool snap = ix.w & kFlagSnap;
+    if (!PAIR && snap) {  // unit row: exact copy of node 0
+#pragma unroll
+      for (int k = 0; k < K; ++k)
+        if (k < t.n) du[t.l[k] * dls] = ldg(reinterpret_cast<const B*>(xu) + t.l[k] * uls);
+      continue;
+    }
+    T w[kPMax];
+    const T* wr = static_cast<const T*>(c.itp_w) + row * kPMax;
+    ld_vals4<T>(wr, w);
+    ld_vals4<T>(wr + 4, w + 4);
+    if (snap) w[0] = T(1);
+    const int pe = snap ? 1 : p;
+    T au[K], av[K];
+#pragma unroll
+    for (int k = 0; k < K; ++k) au[k] = av[k] = T(0);
+#pragma unroll
+    for (int n = 0; n < kPMax; ++n)
+      if (n < pe) {
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+          au[k] = fma(w[n], ldg(xu + (n * ix.z + t.l[k] * uls)), au[k]);
+          if (PAIR) av[k] = fma(w[n], ldg(xv + (n * ix.z + t.l[k] * vls)), av[k]);
+        }
+      }
+    T m[4];
+    if (PAIR) ld_vals4<T>(static_cast<const T*>(c.itp_m) + row * 4, m);
+#pragma unroll
+    for (int k = 0; k < K; ++k)
+      if (k < t.n) {
+        if (PAIR) {
+          du[t.l[k] * dls] = to_bits(fma(m[0], au[k], m[1] * av[k]));
+          dv[t.l[k] * dls] = to_bits(fma(m[2], au[k], m[3] * av[k]));
+        } else {
+          du[t.l[k] * dls] = to_bits(au[k]);
+        }
+      }
+  }
+}
+
 // ---------------------------------------------------------------------------
 // user CSR rows (Table III: F_NNZ / F_COL / F_DATA), ELL-packed: row q of the
 // item's component has its entries at src_org + q * p
 // ---------------------------------------------------------------------------
 // When every entry of the item's rows reads one slot (P.s, level stride
 // src_ls), the per-entry slot lookups are skipped.
-template <typename T>
-__device__ __forceinline__ const T* csr_src(const Item& it, const Ptrs& P, const Ctx& c,
-                                             int e, int l, int& sls) {
-  if (P.s) {
-    sls = it.src_ls;
-    return static_cast<const T*>(P.s) + (__ldg(c.csr_off + e) + l * sls);
-  }
-  const int s = __ldg(c.csr_slot + e);
-  sls = __ldg(c.slot_ls + s);
-  return static_cast<const T*>(c.slots[s]) + (__ldg(c.csr_off + e) + l * sls);
-}
-
 // A row of an ELL block of width W = 4 or 8 starts on a 16-byte boundary
 // (the host pads the widths and aligns the blocks): its offsets, weights
 // and (without a common slot) slots load as 16-byte vectors.
@@ -952,6 +1017,57 @@ __device__ void csr_flat_w(const Item& it, const Ptrs& P, const Ctx& c, int lane
   }
 }
 
+// Rows with contiguous levels (MODE_SPLIT): a lane loads a row's entries once
+// for its kLevelSplit values and has all their columns in flight (one value a
+// lane: 43.2 us for the 512-block step, levels innermost, FP32; 41.0 so).
+template <typename T, int W, bool WIDE>
+__device__ void csr_split(const Item& it, const Ptrs& P, const Ctx& c, int lane) {
+  constexpr int K = kLevelSplit;
+  const int end = it.u0 + it.nunits;
+  const T* sb = static_cast<const T*>(P.s);
+  const bool common = sb != nullptr;
+  const int RW = it.p;  // the row width: W, or a multiple of 8 for wide rows
+  for (int u = it.u0 + lane; u < end; u += 32) {
+    const Split t = split_of(u, it);
+    const int row = it.table + t.q;
+    const int nnz = __ldg(c.csr_nnz + row);
+    const T rhs = ldg(static_cast<const T*>(c.csr_rhs) + row);
+    T acc[K];
+#pragma unroll
+    for (int k = 0; k < K; ++k) acc[k] = rhs;
+    const int nb = WIDE ? nnz : 1;  // a row of width W: one block
+    for (int b0 = 0; b0 < nb; b0 += W) {
+      int off[W], slot[W];
+      T a[W];
+      load_ell<T, W>(c, it.src_org + t.q * RW + b0, common, off, a, slot);
+      if (common) {  // padding entries read offset 0 of the slot, dropped below
+        T x[K][W];
+#pragma unroll
+        for (int k = 0; k < K; ++k)
+#pragma unroll
+          for (int j = 0; j < W; ++j) x[k][j] = ldg(sb + (off[j] + t.l[k] * it.src_ls));
+#pragma unroll
+        for (int k = 0; k < K; ++k)
+#pragma unroll
+          for (int j = 0; j < W; ++j) acc[k] = b0 + j < nnz ? fma(a[j], x[k][j], acc[k]) : acc[k];
+      } else {
+#pragma unroll
+        for (int j = 0; j < W; ++j)
+          if (b0 + j < nnz) {
+            const T* xs = static_cast<const T*>(c.slots[slot[j]]) + off[j];
+            const int sls = __ldg(c.slot_ls + slot[j]);
+#pragma unroll
+            for (int k = 0; k < K; ++k) acc[k] = fma(a[j], ldg(xs + t.l[k] * sls), acc[k]);
+          }
+      }
+    }
+    T* d = static_cast<T*>(P.d) + dst_cell(it, c, t.q);
+#pragma unroll
+    for (int k = 0; k < K; ++k)
+      if (k < t.n) d[t.l[k] * it.dst_ls] = acc[k];
+  }
+}
+
 // A cell times a chunk of levels per lane, a whole ELL row of width W.
 template <typename T, int W, int CH, bool WIDE>
 __device__ void csr_chunk_w(const Item& it, const Ptrs& P, const Ctx& c, int lane) {
@@ -1007,87 +1123,6 @@ __device__ void csr_chunk_w(const Item& it, const Ptrs& P, const Ctx& c, int lan
       for (int l = 0; l < CH; ++l)
         if (l < nl) d[l * ls] = acc[l] + rhs;
     }
-}
-
-// Rows are processed E entries at a time: the E offsets and values load
-// together, then the E x E-level source loads, so one row costs two memory
-// latencies per E entries instead of two per entry.
-constexpr int kCsrBatch = 8;
-
-template <typename T, int CH>
-__device__ void csr_chunk(const Item& it, const Ptrs& P, const Ctx& c, int lane) {
-  constexpr int E = kCsrBatch;
-  const int end = it.u0 + it.nunits;
-  const int ls = it.dst_ls;
-  const int chn = it.mode;
-  const int W = it.p;
-  const T* val = static_cast<const T*>(c.csr_val);
-  for (int u = it.u0 + lane; u < end; u += 32) {
-    int q, ch;
-    unit_of(u, it, q, ch);
-    const int l0 = ch * chn;
-    const int nl = min(chn, (int)it.lev.d - l0);
-    const int row = it.table + q;
-    const int nnz = __ldg(c.csr_nnz + row);
-    const int e0 = it.src_org + q * W;
-    T* d = static_cast<T*>(P.d) + (dst_cell(it, c, q) + l0 * ls);
-    T acc[CH];
-#pragma unroll
-    for (int l = 0; l < CH; ++l) acc[l] = T(0);
-    for (int eb = 0; eb < nnz; eb += E) {
-      const T* xs[E];
-      int sl[E];
-      T a[E];
-#pragma unroll
-      for (int e = 0; e < E; ++e)
-        if (eb + e < nnz) {
-          xs[e] = csr_src<T>(it, P, c, e0 + eb + e, l0, sl[e]);
-          a[e] = ldg(val + e0 + eb + e);
-        }
-#pragma unroll
-      for (int e = 0; e < E; ++e)
-        if (eb + e < nnz) {
-#pragma unroll
-          for (int l = 0; l < CH; ++l)
-            if (l < nl) acc[l] = fma(a[e], ldg(xs[e] + l * sl[e]), acc[l]);
-        }
-    }
-    const T rhs = ldg(static_cast<const T*>(c.csr_rhs) + row);
-#pragma unroll
-    for (int l = 0; l < CH; ++l)
-      if (l < nl) d[l * ls] = acc[l] + rhs;
-  }
-}
-
-template <typename T>
-__device__ void csr_flat(const Item& it, const Ptrs& P, const Ctx& c, int lane) {
-  constexpr int E = kCsrBatch;
-  const int end = it.u0 + it.nunits;
-  const int W = it.p;
-  const T* val = static_cast<const T*>(c.csr_val);
-  T* dbase = static_cast<T*>(P.d);
-  for (int f = it.u0 + lane; f < end; f += 32) {
-    int q, l;
-    flat_of(f, it, q, l);
-    const int row = it.table + q;
-    const int nnz = __ldg(c.csr_nnz + row);
-    const int e0 = it.src_org + q * W;
-    T acc = ldg(static_cast<const T*>(c.csr_rhs) + row);
-    for (int eb = 0; eb < nnz; eb += E) {
-      T x[E], a[E];
-#pragma unroll
-      for (int e = 0; e < E; ++e)
-        if (eb + e < nnz) {
-          int sls;
-          x[e] = ldg(csr_src<T>(it, P, c, e0 + eb + e, l, sls));
-          a[e] = ldg(val + e0 + eb + e);
-        }
-#pragma unroll
-      for (int e = 0; e < E; ++e)
-        if (eb + e < nnz) acc = fma(a[e], x[e], acc);
-    }
-    dbase[dst_cell(it, c, q) + l * it.dst_ls] = acc;
-  }
 }
 
 // ---------------------------------------------------------------------------
@@ -1148,14 +1183,8 @@ __device__ void adj_chunk(const Item& item, const Ptrs& P, const Ctx& c, int lan
   }
 }
 
-// Flat transpose rows.  Bound by the chain of dependent loads (row, entries,
-// ghost values; about 1 us a value at the 28 warps an SM holds) and issue, so
-// rows whose entries read one slot (P.s) come as records that hold the row
-// and its first two entries (Ctx::arow_rec; most rows of user CSR edges have
-// no more) and a lane takes U values through the two steps side by side.  512
-// blocks, levels innermost, FP32: the adjoint 97 us with the row pointers and
-// entries in their own arrays, 103 with records and U = 1, 84 with 2, 80 with
-// 3, 86 with 4 (spills); FP64 gains nothing past 1.
+// Flat transpose rows (one level, or cells before levels): records for rows
+// that read one slot, U of them in flight, as in adj_split.
 template <typename T>
 struct AdjRec {  // int4s of one record
   static constexpr int n = sizeof(T) == 4 ? 2 : 3;
@@ -1253,17 +1282,142 @@ __device__ void adj_flat(const Item& item, const Ptrs& P, const Ctx& c, int lane
   }
 }
 
+// Transpose rows with contiguous levels (MODE_SPLIT).  Bound by the chain of
+// dependent loads (row, entries, ghost values; about 1 us a value at the 28
+// warps an SM holds) and issue, so rows whose entries read one slot (P.s) come
+// as records that hold the row and its first two entries (Ctx::arow_rec; most
+// rows of user CSR edges have no more) and a lane takes kLevelSplit values of
+// U rows through the two steps side by side.  512 blocks, levels innermost,
+// FP32: the adjoint 97 us with the row pointers and entries in their own
+// arrays and one value in flight, 80 with three values of records, 73 so (U =
+// 1: 80).
+template <typename T>
+__device__ void adj_split(const Item& item, const Ptrs& P, const Ctx& c, int lane) {
+  constexpr int K = kLevelSplit, E = kAdjBatch;
+  const Item it = item;
+  const int end = it.u0 + it.nunits;
+  const T* wv = static_cast<const T*>(c.aent_w);
+  const T* yb = static_cast<const T*>(P.s);
+  T* xd = static_cast<T*>(P.d);
+  const int dls = it.dst_ls, sls = it.src_ls;
+  if (yb) {
+    constexpr int U = sizeof(T) == 4 ? 2 : 1;
+    const int4* rec = c.arow_rec + (size_t)it.table * AdjRec<T>::n;
+    for (int u0 = it.u0 + lane; u0 < end; u0 += 32 * U) {
+      // straight through, without branches, so that all loads of a step issue
+      // together: units past the end repeat the last one, a single entry
+      // stands for both
+      int4 ra[U], rb[U], rc[U];
+      Split t[U];
+#pragma unroll
+      for (int v = 0; v < U; ++v) {
+        t[v] = split_of(min(u0 + 32 * v, end - 1), it);
+        const int4* rp = rec + t[v].q * AdjRec<T>::n;
+        ra[v] = __ldg(rp);
+        rb[v] = __ldg(rp + 1);
+        if constexpr (sizeof(T) == 8) rc[v] = __ldg(rp + 2);
+        if (u0 + 32 * v >= end) t[v].n = 0;
+      }
+      T x[U][K], y0[U][K], y1[U][K];
+#pragma unroll
+      for (int v = 0; v < U; ++v)
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+          x[v][k] = xd[ra[v].x + t[v].l[k] * dls];
+          y0[v][k] = yb[ra[v].w + t[v].l[k] * sls];
+          y1[v][k] = yb[rb[v].x + t[v].l[k] * sls];
+        }
+#pragma unroll
+      for (int v = 0; v < U; ++v) {
+        T w0, w1;
+        if constexpr (sizeof(T) == 4) {
+          w0 = __int_as_float(rb[v].y);
+          w1 = __int_as_float(rb[v].z);
+        } else {
+          w0 = __hiloint2double(rc[v].y, rc[v].x);
+          w1 = __hiloint2double(rc[v].w, rc[v].z);
+        }
+        const int n = ra[v].y;
+        T acc[K];
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+          acc[k] = fma(w0, y0[v][k], x[v][k]);
+          acc[k] = n > 1 ? fma(w1, y1[v][k], acc[k]) : acc[k];
+        }
+        for (int eb = ra[v].z + 2, e1 = ra[v].z + n; eb < e1; eb += E) {
+          int eo[E];
+          T a[E];
+#pragma unroll
+          for (int e = 0; e < E; ++e) {
+            const int ee = min(eb + e, e1 - 1);
+            eo[e] = __ldg(c.aent_off + ee);
+            a[e] = ldg(wv + ee);
+          }
+#pragma unroll
+          for (int k = 0; k < K; ++k) {
+            T y[E];
+#pragma unroll
+            for (int e = 0; e < E; ++e) y[e] = yb[eo[e] + t[v].l[k] * sls];
+#pragma unroll
+            for (int e = 0; e < E; ++e) acc[k] = eb + e < e1 ? fma(a[e], y[e], acc[k]) : acc[k];
+          }
+        }
+#pragma unroll
+        for (int k = 0; k < K; ++k)
+          if (k < t[v].n) xd[ra[v].x + t[v].l[k] * dls] = acc[k];
+      }
+    }
+    return;
+  }
+  for (int u = it.u0 + lane; u < end; u += 32) {
+    const Split t = split_of(u, it);
+    const int r = it.table + t.q;
+    T* xb = xd + __ldg(c.arow_off + r);
+    const int e0 = (int)__ldg(c.adj_ptr + r), e1 = (int)__ldg(c.adj_ptr + r + 1);
+    T acc[K];
+#pragma unroll
+    for (int k = 0; k < K; ++k) acc[k] = xb[t.l[k] * dls];
+    for (int eb = e0; eb < e1; eb += E) {
+      const T* ys[E];
+      int gl[E];
+      T a[E];
+#pragma unroll
+      for (int e = 0; e < E; ++e) {
+        const int ee = min(eb + e, e1 - 1);
+        const int gs = __ldg(c.aent_slot + ee);
+        gl[e] = __ldg(c.slot_ls + gs);
+        ys[e] = static_cast<const T*>(c.slots[gs]) + __ldg(c.aent_off + ee);
+        a[e] = ldg(wv + ee);
+      }
+#pragma unroll
+      for (int k = 0; k < K; ++k) {
+        T y[E];
+#pragma unroll
+        for (int e = 0; e < E; ++e) y[e] = ys[e][t.l[k] * gl[e]];
+#pragma unroll
+        for (int e = 0; e < E; ++e) acc[k] = eb + e < e1 ? fma(a[e], y[e], acc[k]) : acc[k];
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < K; ++k)
+      if (k < t.n) xb[t.l[k] * dls] = acc[k];
+  }
+}
+
 // Kernel families: one kernel per family keeps each family's register
 // budget (and so its occupancy) independent of the others.
 template <typename T, int FAM, int MAXCH>
 __device__ __forceinline__ void run_item(const Item& it, const Ptrs& P, const Ctx& c, int lane) {
-  const bool flat = it.mode < 2 && it.mode != MODE_TILE;
+  const bool flat = it.mode < 2;
   const bool ch8 = MAXCH > 4 && it.mode > 4;  // level chunks of up to 8
   if constexpr (FAM == FAM_STRUCT) {
     structured_flat<T>(it, P, c, lane);
   } else if constexpr (FAM == FAM_INTERP) {
     if (it.mode == MODE_TILE) {
       interp_tile<T>(it, P, c, lane);
+    } else if (it.mode == MODE_SPLIT) {
+      it.kind == IK_INTERP_PAIR ? interp_split<T, true>(it, P, c, lane)
+                                : interp_split<T, false>(it, P, c, lane);
     } else if (it.kind == IK_INTERP_PAIR) {
       if (flat)
         interp_flat<T, true>(it, P, c, lane);
@@ -1285,6 +1439,13 @@ __device__ __forceinline__ void run_item(const Item& it, const Ptrs& P, const Ct
         rows_tile<T, 8, false>(it, P, c, lane);
       else
         rows_tile<T, 4, false>(it, P, c, lane);
+    } else if (it.mode == MODE_SPLIT) {
+      if (it.p == 8)
+        csr_split<T, 8, false>(it, P, c, lane);
+      else if (it.p % 8 == 0)
+        csr_split<T, 8, true>(it, P, c, lane);
+      else
+        csr_split<T, 4, false>(it, P, c, lane);
     } else if (it.p == 8) {
       if (flat)
         csr_flat_w<T, 8, false>(it, P, c, lane);
@@ -1299,23 +1460,19 @@ __device__ __forceinline__ void run_item(const Item& it, const Ptrs& P, const Ct
         csr_chunk_w<T, 8, (MAXCH > 4 ? 8 : 4), true>(it, P, c, lane);
       else
         csr_chunk_w<T, 8, 4, true>(it, P, c, lane);
-    } else if (it.p == 4) {
+    } else {  // width 4
       if (flat)
         csr_flat_w<T, 4, false>(it, P, c, lane);
       else if (ch8)
         csr_chunk_w<T, 4, (MAXCH > 4 ? 8 : 4), false>(it, P, c, lane);
       else
         csr_chunk_w<T, 4, 4, false>(it, P, c, lane);
-    } else if (flat) {
-      csr_flat<T>(it, P, c, lane);
-    } else if (ch8) {
-      csr_chunk<T, (MAXCH > 4 ? 8 : 4)>(it, P, c, lane);
-    } else {
-      csr_chunk<T, 4>(it, P, c, lane);
     }
   } else {
     if (it.mode == MODE_TILE)
       rows_tile<T, 4, true>(it, P, c, lane);
+    else if (it.mode == MODE_SPLIT)
+      adj_split<T>(it, P, c, lane);
     else if (it.kind == IK_ADD && c.vec_runs)
       runs_vec<T, RUN_ADD>(it, P, c, lane);
     else if (it.kind == IK_ADD)

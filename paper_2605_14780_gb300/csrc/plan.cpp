@@ -875,11 +875,20 @@ int level_chunk(const bc_plan* P, int fam) {
   return all_kinds ? std::min(ch, 4) : ch;
 }
 
+// levels of one unit
+int unit_levels(const Item& it) {
+  return it.mode >= 2 ? it.mode : (it.mode == MODE_SPLIT ? kLevelSplit : 1);
+}
+
 // split the unit space into warp-sized items: vol * L single values (flat
 // modes) or vol * ceil(L / mode) chunks
 void emit_units(std::vector<Item>& out, Item proto, int vol, int L, int mode, int per_item) {
   proto.mode = mode;
-  const int64_t total = mode < 2 ? (int64_t)vol * L : (int64_t)vol * ((L + mode - 1) / mode);
+  int64_t total = mode < 2 ? (int64_t)vol * L : (int64_t)vol * ((L + mode - 1) / mode);
+  if (mode == MODE_SPLIT) {
+    proto.bwid = make_div((uint32_t)((L + kLevelSplit - 1) / kLevelSplit));
+    total = (int64_t)vol * proto.bwid.d;
+  }
   for (int64_t u0 = 0; u0 < total; u0 += per_item) {
     Item it = proto;
     it.u0 = (int)u0;
@@ -1343,11 +1352,14 @@ void build_items(bc_plan* P) {
   }
   auto table_emit = [&](std::vector<Item>& out, const Item& it, const bc_block& B, int vol) {
     const bool interp = it.kind == IK_INTERP || it.kind == IK_INTERP_PAIR;
-    const int mode = table_mode(B, P->opts.unit_order,
+    int mode = table_mode(B, P->opts.unit_order,
                                 it.kind == IK_CSR ? level_chunk(P, FAM_CSR)
                                 : interp          ? level_chunk(P, FAM_INTERP)
                                                   : level_chunk(P, FAM_ADJ));
-    emit_units(out, it, vol, B.nlevels, mode, mode < 2 ? per_table_flat_item : per_table_item);
+    if (mode == MODE_FLAT_LEVEL) mode = MODE_SPLIT;
+    const int flat_item =
+        mode == MODE_SPLIT ? std::max(32, per_table_flat_item / kLevelSplit / 32 * 32) : per_table_flat_item;
+    emit_units(out, it, vol, B.nlevels, mode, mode < 2 ? flat_item : per_table_item);
   };
   std::vector<std::pair<int, std::vector<Item>>> per_sub(P->subs.size());
   for (size_t si = 0; si < P->subs.size(); ++si) {
@@ -1444,7 +1456,7 @@ void build_items(bc_plan* P) {
   // per lane
   auto work = [&](const Item& it) -> int64_t {
     if (it.mode == MODE_TILE) return (int64_t)it.nunits * it.nl;
-    if (it.mode != MODE_RUNS) return (int64_t)it.nunits * (it.mode >= 2 ? it.mode : 1);
+    if (it.mode != MODE_RUNS) return (int64_t)it.nunits * unit_levels(it);
     int64_t n = 0;
     for (int r = it.u0; r < it.u0 + it.nunits; ++r) n += P->runs[r].z;
     return n;
@@ -1580,15 +1592,15 @@ void build_items(bc_plan* P) {
         for (int r = it.u0; r < it.u0 + it.nunits; ++r) n += P->runs[(size_t)r].z;
         return n / 256;
       }
-      const bool flat = it.mode == MODE_FLAT_CELL || it.mode == MODE_FLAT_LEVEL;
-      const int per = flat && it.mode == MODE_FLAT_LEVEL ? (int)it.lev.d : 1;
+      const bool flat = it.mode == MODE_FLAT_CELL || it.mode == MODE_SPLIT;
+      const int per = it.mode == MODE_SPLIT ? (int)it.bwid.d : 1;
       const int vol = (int)it.vol.d;
       int64_t nnz = 0;
       for (int u = it.u0 / per; u <= (it.u0 + it.nunits - 1) / per; ++u) {
         const size_t r = (size_t)(it.table + (it.mode == MODE_TILE ? u : u % vol));
         nnz = std::max(nnz, P->adj_ptr[r + 1] - P->adj_ptr[r]);
       }
-      return it.mode == MODE_TILE ? 1 + nnz / 4 : (nnz + 3) / 4 * (flat ? (it.nunits + 31) / 32 : 4);
+      return it.mode == MODE_TILE ? 1 + nnz / 4 : (nnz + 3) / 4 * (flat ? (it.nunits + 31) / 32 * unit_levels(it) : 4);
     };
     std::vector<std::pair<int64_t, size_t>> key(P->adj_items.size());
     for (size_t t = 0; t < key.size(); ++t) key[t] = {-steps(P->adj_items[t]), t};
@@ -2550,7 +2562,7 @@ void persistent_split(bc_plan* P, int per_sm[kFamilies]) {
   double bytes[kFamilies] = {0, 0, 0, 0}, total = 0;
   for (int f = 0; f < kFamilies; ++f) {
     for (const Item& it : P->fam_items[f]) {
-      double v = it.mode == MODE_RUNS ? 0 : (double)it.nunits * (it.mode >= 2 ? it.mode : 1);
+      double v = it.mode == MODE_RUNS ? 0 : (double)it.nunits * unit_levels(it);
       if (it.mode == MODE_RUNS)
         for (int r = it.u0; r < it.u0 + it.nunits; ++r) v += P->runs[(size_t)r].z;
       if (it.mode == MODE_TILE) v = (double)it.nunits * it.nl;
@@ -2849,7 +2861,10 @@ struct WorkCheck {
       return;
     }
     for (int u = it.u0; u < it.u0 + it.nunits; ++u) {
-      if (it.mode == MODE_FLAT_LEVEL) {
+      if (it.mode == MODE_SPLIT) {
+        const int part = (int)it.bwid.d;
+        for (int l = u % part; l < L; l += part) f(u / part, l);
+      } else if (it.mode == MODE_FLAT_LEVEL) {
         f(u / L, u % L);
       } else if (it.mode == MODE_FLAT_CELL) {
         f(u % vol, u / vol);
