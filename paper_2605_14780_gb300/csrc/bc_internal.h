@@ -312,6 +312,9 @@ struct SyncCtx {
   int level_fast = 0;   // 1: consecutive threads take consecutive levels
                         //    (levels contiguous in memory), 0: consecutive
                         //    rows at one level
+  // closed groups of rows (ngroups 0: none): up to four rows, -1 past the last
+  int ngroups = 0;
+  const int4* group = nullptr;
   const int4* row = nullptr;
   const int32_t* ptr = nullptr;
   const int2* ent = nullptr;
@@ -326,7 +329,8 @@ enum SyncStep : int32_t {
   SYNC_ROWS = 0,      // stage = A_sync x (reads data)
   SYNC_COMMIT = 1,    // data = stage
   SYNC_SNAPSHOT = 2,  // stage = y_bar of the Sync rows, then y_bar = 0
-  SYNC_ADJOINT = 3    // x_bar += A_sync^T stage
+  SYNC_ADJOINT = 3,   // x_bar += A_sync^T stage
+  SYNC_GROUPS = 4     // closed groups: data = A_sync x, in place
 };
 cudaError_t launch_sync(int dtype, int step, const SyncCtx& s, void* const* slots,
                         const int32_t* slot_ls, cudaStream_t stream);

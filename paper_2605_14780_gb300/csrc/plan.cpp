@@ -189,6 +189,7 @@ struct bc_plan {
     std::vector<int32_t> cstage;
     std::vector<double> cw;
     int64_t stage = 0;  // staging values (rows x levels)
+    std::vector<int4> group;  // closed groups of rows, when all rows are in one
   } sync;
   SyncCtx sync_ctx{};
   // work lists
@@ -603,6 +604,48 @@ bc_status add_sync(bc_plan* P, const bc_submatrix& m, int idx, Coverage& dcov) {
   }
   if (P->sync.stage > INT32_MAX) return fail(BC_ERR_UNSUPPORTED, "too many Sync values");
   return BC_OK;
+}
+
+// Groups of at most four Sync rows that read exactly the cells they write;
+// none when some row is in no such group.
+void build_sync_groups(bc_plan* P) {
+  auto& S = P->sync;
+  S.group.clear();
+  const size_t n = S.row.size();
+  std::unordered_map<int64_t, int32_t> row_of;
+  for (size_t r = 0; r < n; ++r) row_of[col_key(S.row[r].x, S.row[r].y)] = (int32_t)r;
+  std::vector<int32_t> up(n);
+  std::iota(up.begin(), up.end(), 0);
+  auto root = [&](int32_t r) {
+    while (up[r] != r) r = up[r] = up[up[r]];
+    return r;
+  };
+  for (size_t r = 0; r < n; ++r)
+    for (int32_t e = S.ptr[r]; e < S.ptr[r + 1]; ++e) {
+      const auto it = row_of.find(col_key(S.ent[e].x, S.ent[e].y));
+      if (it == row_of.end()) return;  // reads a cell that no row writes
+      const int32_t a = root((int32_t)r), b = root(it->second);
+      if (a != b) up[std::max(a, b)] = std::min(a, b);
+    }
+  // groups in the order of their first rows, rows ascending
+  std::vector<int32_t> group_of(n, -1);
+  std::vector<int4> groups;
+  for (size_t r = 0; r < n; ++r) {
+    int32_t& g = group_of[root((int32_t)r)];
+    if (g < 0) {
+      g = (int32_t)groups.size();
+      groups.push_back(make_int4((int)r, -1, -1, -1));
+    } else if (groups[g].y < 0) {
+      groups[g].y = (int)r;
+    } else if (groups[g].z < 0) {
+      groups[g].z = (int)r;
+    } else if (groups[g].w < 0) {
+      groups[g].w = (int)r;
+    } else {
+      return;
+    }
+  }
+  S.group.swap(groups);
 }
 
 // Columns read by Sync rows and their entries {staging offset, weight}, in
@@ -1863,6 +1906,7 @@ bc_status upload_tables(bc_plan* P) {
   const size_t o_ew = L.take(P->aent_w.size() * S);
   const auto& Y = P->sync;
   const size_t o_yr = L.take(Y.row.size() * sizeof(int4));
+  const size_t o_yg = L.take(Y.group.size() * sizeof(int4));
   const size_t o_yp = L.take(Y.ptr.size() * 4);
   const size_t o_ye = L.take(Y.ent.size() * sizeof(int2));
   const size_t o_yw = L.take(Y.w.size() * S);
@@ -1874,6 +1918,7 @@ bc_status upload_tables(bc_plan* P) {
   const size_t o_ctr = L.take(kCtrWords * kFamilies * kCounterStreams * sizeof(unsigned));  // zero
   std::vector<char> host(L.off + 256, 0);
   put_raw(host, o_yr, Y.row);
+  put_raw(host, o_yg, Y.group);
   put_raw(host, o_yp, Y.ptr);
   put_raw(host, o_ye, Y.ent);
   put_raw(host, o_yc, Y.col);
@@ -1950,6 +1995,8 @@ bc_status upload_tables(bc_plan* P) {
     if (r.w > 1 && P->slot_ls[r.x] != 1) y.level_fast = 0;
   }
   y.row = reinterpret_cast<const int4*>(b + o_yr);
+  y.ngroups = (int)Y.group.size();
+  y.group = reinterpret_cast<const int4*>(b + o_yg);
   y.ptr = reinterpret_cast<const int32_t*>(b + o_yp);
   y.ent = reinterpret_cast<const int2*>(b + o_ye);
   y.w = b + o_yw;
@@ -2082,7 +2129,7 @@ void compute_stats(bc_plan* P) {
   st.batch_mode = P->opts.batch_mode;
   st.level_chunk = P->opts.level_chunk;
   const int ys = P->sync_ctx.nrows > 0 ? 2 : 0;
-  st.launches_fwd = ys;
+  st.launches_fwd = P->sync_ctx.ngroups > 0 ? 1 : ys;
   if (P->opts.batch_mode == BC_BATCH_PERSISTENT || P->opts.batch_mode == BC_BATCH_SINGLE)
     st.launches_fwd += P->all_items.empty() ? 0 : 1;
   else
@@ -2424,6 +2471,7 @@ bc_status plan_create_impl(const bc_grid* grid, const bc_submatrix* subs, int32_
     for (int si : syn)
       if ((st = add_sync(P, subs[si], si, dcov)) != BC_OK) return st;
     build_sync_transpose(P);
+    build_sync_groups(P);
   }
   // cell tables: every box cell's offset, and the source cell of maps
   for (Sub& s2 : P->subs) {
@@ -2590,7 +2638,8 @@ bc_status launch_forward(bc_plan* P, void* const* slots, int form, cudaStream_t 
   // Sync rows read the input data: evaluate them into the staging buffer
   // while the ghost kernels run (they write only ghosts), write them back
   // after every kernel that reads data has run
-  const bool sync = P->sync_ctx.nrows > 0;
+  // (rows in closed groups are summed in place after those kernels instead)
+  const bool sync = P->sync_ctx.nrows > 0 && P->sync_ctx.ngroups == 0;
   if (sync && form != BC_FORM_BATCHED &&
       (e = launch_sync(P->dtype, SYNC_ROWS, P->sync_ctx, slots, c.slot_ls, s)) != cudaSuccess)
     return cuda_fail(e, "Sync rows");
@@ -2653,7 +2702,8 @@ bc_status launch_forward(bc_plan* P, void* const* slots, int form, cudaStream_t 
   } else {
     return fail(BC_ERR_INVALID_ARG, "unknown form %d", form);
   }
-  if (e == cudaSuccess) e = launch_sync(P->dtype, SYNC_COMMIT, P->sync_ctx, slots, c.slot_ls, s);
+  if (e == cudaSuccess)
+    e = launch_sync(P->dtype, sync ? SYNC_COMMIT : SYNC_GROUPS, P->sync_ctx, slots, c.slot_ls, s);
   if (e != cudaSuccess) return cuda_fail(e, "forward launch");
   return BC_OK;
 }
@@ -3720,6 +3770,23 @@ int64_t check_sync(WorkCheck& W) {
     for (int32_t e = Y.ptr[u]; e < Y.ptr[u + 1]; ++e)
       want[col_key(Y.ent[(size_t)e].x, Y.ent[(size_t)e].y)].push_back({r.z, Y.w[(size_t)e]});
   }
+  // closed groups: every row in one group, reading only cells its group writes
+  std::vector<int> grouped(Y.row.size(), 0);
+  for (const int4& g : Y.group) {
+    const int rows[4] = {g.x, g.y, g.z, g.w};
+    std::unordered_set<int64_t> cells;
+    for (int r : rows)
+      if (r >= 0) {
+        ++grouped[(size_t)r];
+        cells.insert(col_key(Y.row[(size_t)r].x, Y.row[(size_t)r].y));
+      }
+    for (int r : rows)
+      for (int32_t e = r >= 0 ? Y.ptr[(size_t)r] : 0; r >= 0 && e < Y.ptr[(size_t)r + 1]; ++e)
+        if (!cells.count(col_key(Y.ent[(size_t)e].x, Y.ent[(size_t)e].y)))
+          W.problem("a Sync group reads a cell it does not write", Y.row[(size_t)r].x, Y.row[(size_t)r].y);
+  }
+  for (size_t r = 0; !Y.group.empty() && r < grouped.size(); ++r)
+    if (grouped[r] != 1) W.problem("a Sync row is not in one group", Y.row[r].x, Y.row[r].y);
   for (size_t i = 0; i < stage_hits.size(); ++i)
     if (stage_hits[i] != 1) W.problem("a staging value is not used exactly once", -1, (int64_t)i);
   for (size_t u = 0; u < Y.col.size(); ++u) {
