@@ -182,9 +182,12 @@ constexpr int FAM_ALL = 4;
 // `threads` per CTA (32..512).  grid <= 0: a plain grid with one warp per
 // item; otherwise `grid` resident CTAs whose warps walk the items with a
 // fixed stride, prefetching the next items' descriptors and slot pointers.
+// grid kGridAfter (FAM_STRUCT only): a plain grid that may start while the
+// kernel before it in the stream still runs; its stores wait for that one.
 // stage: bytes of one warp's shared-memory stage that the list's staged
 // tiles (MODE_TILE) need (kStageBytesRows or kStageBytesCsr), 0 when it has
 // none: the launch requests that much dynamic shared memory per warp.
+constexpr int kGridAfter = -1;
 cudaError_t launch_family(int dtype, int family, const Ctx& ctx,
                           const Item* items, int nitems, int threads, int grid,
                           int stage, cudaStream_t s);

@@ -1587,6 +1587,10 @@ __global__ void __launch_bounds__(THREADS, (Occ<FAM, THREADS>::kMinBlocks))
   Ptrs P = gather_ptrs(lookup_slot(c, w, lane));
   if (Stage<FAM, THREADS>::kWarps) P.stage = warp * c.stage_warp;
   __syncwarp();
+  // the adjoint's zero pass starts while the gather's last CTAs run
+  // (launch_after): it reads its items by then, and stores after the gather
+  if constexpr (FAM == FAM_STRUCT) asm volatile("griddepcontrol.wait;\n" ::: "memory");
+  if constexpr (FAM == FAM_ADJ) asm volatile("griddepcontrol.launch_dependents;\n");
   run_work<T, FAM>(sit[warp], P, c, lane);
 }
 
@@ -1714,6 +1718,21 @@ cudaError_t launch_t(const Ctx& c, const Item* items, int nitems, int grid, int 
                      cudaStream_t s) {
   const int wpb = THREADS / 32;
   const int need = (nitems + wpb - 1) / wpb;
+  if (grid == kGridAfter) {
+    // programmatic dependent launch on the kernel before it in the stream
+    if constexpr (FAM == FAM_STRUCT) {
+      cudaLaunchConfig_t cfg{};
+      cfg.gridDim = dim3((unsigned)need);
+      cfg.blockDim = dim3(THREADS);
+      cfg.stream = s;
+      cudaLaunchAttribute at{};
+      at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+      at.val.programmaticStreamSerializationAllowed = 1;
+      cfg.attrs = &at;
+      cfg.numAttrs = 1;
+      return cudaLaunchKernelEx(&cfg, k_items<T, THREADS, FAM>, c, items, nitems);
+    }
+  }
   if (grid <= 0) {
     const int smem = stage_smem<FAM, THREADS>(k_items<T, THREADS, FAM>, stage);
     k_items<T, THREADS, FAM><<<need, THREADS, smem, s>>>(c, items, nitems);
