@@ -160,11 +160,29 @@ def _ptr(arr, ctype):
     return arr.ctypes.data_as(ctypes.POINTER(ctype))
 
 
+_CURRENT_STREAM = None
+
+
+def _current_stream():
+    """A function giving the current device's current stream as an integer.
+    ``torch.cuda.current_stream()`` builds a Stream object (3.1 us a call, of
+    6.8 for a small ghost fill); the raw query takes 0.2 us."""
+    import torch
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    if raw is None:
+        return lambda: int(torch.cuda.current_stream().cuda_stream)
+    device = torch.cuda.current_device
+    return lambda: raw(device())
+
+
 def _stream_handle(stream):
-    if stream is None:
-        import torch
-        stream = torch.cuda.current_stream()
-    return ctypes.c_void_p(int(stream.cuda_stream))
+    """The stream's handle (``None``: the current stream) for the library."""
+    if stream is not None:
+        return int(stream.cuda_stream)
+    global _CURRENT_STREAM
+    if _CURRENT_STREAM is None:
+        _CURRENT_STREAM = _current_stream()
+    return _CURRENT_STREAM()
 
 
 class Plan:
@@ -378,12 +396,15 @@ class Plan:
     def apply(self, slot_table, form=BC_FORM_BATCHED, stream=None):
         """Forward apply; ``slot_table`` is a device int64 tensor of slot
         pointers (see :func:`slot_table`)."""
-        _check(self._lib.bc_apply_form(self._h, c_vp(slot_table.data_ptr()),
-                                       int(form), _stream_handle(stream)))
+        st = self._lib.bc_apply_form(self._h, slot_table.data_ptr(), int(form),
+                                     _stream_handle(stream))
+        if st:
+            _check(st)
 
     def adjoint(self, slot_table, stream=None):
-        _check(self._lib.bc_apply_adjoint(self._h, c_vp(slot_table.data_ptr()),
-                                          _stream_handle(stream)))
+        st = self._lib.bc_apply_adjoint(self._h, slot_table.data_ptr(), _stream_handle(stream))
+        if st:
+            _check(st)
 
     def apply_stencil(self, slot_table, out_table, offsets, coeffs, stream=None):
         """Ghost fill fused with the stencil ``sum_p coeffs[p] f(x +
@@ -460,8 +481,10 @@ class Pack:
         self.size = int(lib.bc_pack_size(handle))
 
     def run(self, slot_table, buffer, stream=None):
-        _check(self._lib.bc_pack_run(self._h, c_vp(slot_table.data_ptr()),
-                                     c_vp(buffer.data_ptr()), _stream_handle(stream)))
+        st = self._lib.bc_pack_run(self._h, slot_table.data_ptr(), buffer.data_ptr(),
+                                   _stream_handle(stream))
+        if st:
+            _check(st)
 
     def close(self):
         if getattr(self, "_h", None):
