@@ -195,7 +195,10 @@ typedef struct bc_grid {
  *              one physical location); rhs must be NULL or zero.  One apply
  *              is one application of A: every row reads the input values, so
  *              Sync rows are computed into a plan-owned staging buffer and
- *              written after all other rows have read the data.  Two Sync
+ *              written after all other rows have read the data (when all of
+ *              them fall into groups of at most four that read exactly the
+ *              cells they write, each group is summed and stored in place
+ *              after those rows instead).  Two Sync
  *              boxes must not share a data cell (BC_ERR_OVERLAP).  Because of
  *              the staging buffer, applies of one plan with Sync rows must
  *              not run concurrently on several streams.

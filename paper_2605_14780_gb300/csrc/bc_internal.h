@@ -185,7 +185,7 @@ constexpr int FAM_ALL = 4;
 // grid kGridAfter (FAM_STRUCT only): a plain grid that may start while the
 // kernel before it in the stream still runs; its stores wait for that one.
 // stage: bytes of one warp's shared-memory stage that the list's staged
-// tiles (MODE_TILE) need (kStageBytesRows or kStageBytesCsr), 0 when it has
+// tiles (MODE_TILE) need (the largest stage_bytes of them), 0 when it has
 // none: the launch requests that much dynamic shared memory per warp.
 constexpr int kGridAfter = -1;
 cudaError_t launch_family(int dtype, int family, const Ctx& ctx,
