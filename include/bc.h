@@ -447,8 +447,8 @@ bc_status bc_apply_host(bc_plan* plan, void* const* host_ptrs,
  * (di, dj, dk), coeffs: npoints FP64 weights (rounded to the plan's dtype),
  * both host memory read during the call (they travel as launch
  * parameters: no allocation, graph-capturable).  Each value's sum runs in
- * the order of the points, except that a full 3 x 3 x 3 box with one weight
- * off the centre (and a centre weight at least as large) is summed axis by
+ * the order of the points, except that in FP64 a full 3 x 3 x 3 box with one
+ * weight off the centre (and a centre weight at least as large) is summed axis by
  * axis.  Needs bc_plan_opts.stencil_fusion = 1 at
  * creation (else BC_ERR_UNSUPPORTED, as for plans with Sync rows);
  * BC_ERR_INVALID_ARG for npoints outside 1..125 or a non-finite weight;

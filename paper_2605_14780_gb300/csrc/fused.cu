@@ -451,8 +451,8 @@ cudaError_t launch_fused_box(int dtype, const FuseCtx& F, const FuseStencil& st,
                              cudaStream_t s) {
   if (nctas <= 0) return cudaSuccess;
   const bool unit = st.a == 1.0 || st.a == -1.0;
-  auto* kernel = dtype == 1 ? (unit ? k_fused_box<double, true> : k_fused_box<double, false>)
-                            : (unit ? k_fused_box<float, true> : k_fused_box<float, false>);
+  if (dtype != 1) return cudaErrorInvalidValue;  // FP64 plans only
+  auto* kernel = unit ? k_fused_box<double, true> : k_fused_box<double, false>;
   kernel<<<(unsigned)nctas, kBoxThreads, 0, s>>>(F, st, slots, outs);
   return cudaGetLastError();
 }

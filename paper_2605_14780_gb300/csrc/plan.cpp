@@ -2331,9 +2331,11 @@ bc_status build_fusion(bc_plan* P) {
 // [-1, 1]^3 once each, one weight a off the centre and a centre weight c0
 // with |c0| >= |a| (the box form adds a x0 to the sum and takes it out again
 // with c0 - a, so its rounding stays within |c0 x0|'s share only then),
-// weights as the kernels hold them (the plan's dtype).
+// weights as the kernels hold them (the plan's dtype).  FP64 only: FP32 is not
+// bound by its multiply-adds, and the separate ghost fill costs more than the
+// box sums save (a small FP32 call 18.3 us in one launch, 26.6 us in two).
 void box_stencil(int dtype, FuseStencil& st) {
-  if (st.n != 27) return;
+  if (st.n != 27 || dtype != BC_F64) return;
   auto held = [&](double v) { return dtype == BC_F64 ? v : (double)(float)v; };
   unsigned seen = 0;
   double a = 0, c0 = 0;
