@@ -269,7 +269,6 @@ constexpr int kBoxPitch = kBoxX + 2, kBoxPlane = kBoxPitch * (kBoxY + 2);
 constexpr int kBoxCtas = 512 / kBoxThreads;  // 16 warps an SM
 
 template <typename T> struct Pair2;
-template <> struct Pair2<float> { using type = float2; };
 template <> struct Pair2<double> { using type = double2; };
 
 // 3 x 3 sums of one staged plane for a thread's 2 x 4 cells; `c`: the
@@ -297,17 +296,11 @@ __device__ __forceinline__ void plane_sums(const T* c, T (&P)[2 * kBoxTy]) {
 }
 
 // by the exponent bits: a floating compare would take the FP64 pipe
-__device__ __forceinline__ bool finite_value(float v) {
-  return (__float_as_uint(v) & 0x7f800000u) != 0x7f800000u;
-}
 __device__ __forceinline__ bool finite_value(double v) {
   return ((unsigned)__double2hiint(v) & 0x7ff00000u) != 0x7ff00000u;
 }
 
 // v, or -v where `flip` holds the sign bit (no FP64 instruction either)
-__device__ __forceinline__ float flip_sign(float v, unsigned flip) {
-  return __uint_as_float(__float_as_uint(v) ^ flip);
-}
 __device__ __forceinline__ double flip_sign(double v, unsigned flip) {
   return __hiloint2double((int)((unsigned)__double2hiint(v) ^ flip), __double2loint(v));
 }

@@ -2330,13 +2330,12 @@ bc_status build_fusion(bc_plan* P) {
 // Whether the stencil is a box (FuseStencil::box): the 27 points of
 // [-1, 1]^3 once each, one weight a off the centre and a centre weight c0
 // with |c0| >= |a| (the box form adds a x0 to the sum and takes it out again
-// with c0 - a, so its rounding stays within |c0 x0|'s share only then),
-// weights as the kernels hold them (the plan's dtype).  FP64 only: FP32 is not
+// with c0 - a, so its rounding stays within |c0 x0|'s share only then).
+// FP64 only: FP32 is not
 // bound by its multiply-adds, and the separate ghost fill costs more than the
 // box sums save (a small FP32 call 18.3 us in one launch, 26.6 us in two).
 void box_stencil(int dtype, FuseStencil& st) {
   if (st.n != 27 || dtype != BC_F64) return;
-  auto held = [&](double v) { return dtype == BC_F64 ? v : (double)(float)v; };
   unsigned seen = 0;
   double a = 0, c0 = 0;
   bool first = true;
@@ -2345,7 +2344,7 @@ void box_stencil(int dtype, FuseStencil& st) {
     if (i < 0 || i > 2 || j < 0 || j > 2 || k < 0 || k > 2) return;
     const int at = (k * 3 + j) * 3 + i;
     seen |= 1u << at;
-    const double c = held(st.c[p]);
+    const double c = st.c[p];
     if (at == 13) {
       c0 = c;
     } else if (first) {
@@ -2355,7 +2354,7 @@ void box_stencil(int dtype, FuseStencil& st) {
       return;
     }
   }
-  const double d = held(c0 - a);
+  const double d = c0 - a;
   if (seen != (1u << 27) - 1 || a == 0 || std::fabs(c0) < std::fabs(a) || !std::isfinite(a) ||
       !std::isfinite(d))
     return;
