@@ -608,9 +608,9 @@ template <typename T>
 __device__ __forceinline__ void cp_async_elem(T* smem, const T* gmem) {
   const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
   if constexpr (sizeof(T) == 4)
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(sa), "l"(gmem));
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(sa), "l"(gmem) : "memory");
   else
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(sa), "l"(gmem));
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(sa), "l"(gmem) : "memory");
 }
 
 __device__ __forceinline__ void cp_async_wait_all() {
