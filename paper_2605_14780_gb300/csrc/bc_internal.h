@@ -94,6 +94,11 @@ constexpr int stage_bytes(bool csr, bool pair_or_adj, int esize) {
                       : stage_levels(esize) * (pair_or_adj ? kPlaneAdj : kPlaneInterp));
 }
 static_assert(kPlaneAdj == 2 * kPlaneInterp, "pairs and transpose tiles stage the same bytes");
+constexpr int most_stage_bytes(int esize) {
+  return stage_bytes(true, false, esize) > stage_bytes(false, true, esize)
+             ? stage_bytes(true, false, esize)
+             : stage_bytes(false, true, esize);
+}
 
 struct alignas(16) Item {
   int32_t kind;

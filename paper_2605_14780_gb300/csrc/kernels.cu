@@ -1563,15 +1563,17 @@ struct Stage {
   static constexpr int kWarps = FAM != FAM_STRUCT ? THREADS / 32 : 0;
 };
 
-// dynamic shared memory of a launch with `stage` bytes per warp (the
-// kernel's limit raised first where that exceeds 48 KB: 512 threads with
-// CSR tiles)
-template <int FAM, int THREADS, typename K>
-int stage_smem(K kernel, int stage) {
-  const int bytes = Stage<FAM, THREADS>::kWarps * stage;
-  if (bytes > 48 * 1024)
-    (void)cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-  return bytes;
+// Dynamic shared memory of a launch with `stage` bytes per warp.  Above 48 KB
+// (FP64 CSR tiles from 256 threads, any tiles at 512) the kernel's limit is
+// raised first, always to the most that any list can ask of it: the limit
+// belongs to the kernel, so a value per launch would let a call on another
+// thread lower it between this call's raise and its launch.
+template <typename T, int FAM, int THREADS, typename K>
+cudaError_t stage_smem(K kernel, int stage, int& bytes) {
+  bytes = Stage<FAM, THREADS>::kWarps * stage;
+  if (bytes <= 48 * 1024) return cudaSuccess;
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              Stage<FAM, THREADS>::kWarps * most_stage_bytes((int)sizeof(T)));
 }
 
 // Plain grid: warp w of CTA b processes item b * warps + w.
@@ -1733,11 +1735,15 @@ cudaError_t launch_t(const Ctx& c, const Item* items, int nitems, int grid, int 
       return cudaLaunchKernelEx(&cfg, k_items<T, THREADS, FAM>, c, items, nitems);
     }
   }
+  int smem = 0;
+  cudaError_t e;
   if (grid <= 0) {
-    const int smem = stage_smem<FAM, THREADS>(k_items<T, THREADS, FAM>, stage);
+    if ((e = stage_smem<T, FAM, THREADS>(k_items<T, THREADS, FAM>, stage, smem)) != cudaSuccess)
+      return e;
     k_items<T, THREADS, FAM><<<need, THREADS, smem, s>>>(c, items, nitems);
   } else {
-    const int smem = stage_smem<FAM, THREADS>(k_stream<T, THREADS, FAM>, stage);
+    if ((e = stage_smem<T, FAM, THREADS>(k_stream<T, THREADS, FAM>, stage, smem)) != cudaSuccess)
+      return e;
     k_stream<T, THREADS, FAM><<<grid < need ? grid : need, THREADS, smem, s>>>(c, items, nitems);
   }
   return cudaGetLastError();
@@ -1746,7 +1752,9 @@ cudaError_t launch_t(const Ctx& c, const Item* items, int nitems, int grid, int 
 template <typename T, int THREADS, int FAM>
 cudaError_t persist_t(const Ctx& c, const Item* items, int nitems, int ctas_per_sm, int sms,
                       unsigned* ctr, int stage, cudaStream_t s) {
-  const int smem = stage_smem<FAM, THREADS>(k_persist<T, THREADS, FAM>, stage);
+  int smem = 0;
+  if (cudaError_t e = stage_smem<T, FAM, THREADS>(k_persist<T, THREADS, FAM>, stage, smem))
+    return e;
   int fit = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fit, k_persist<T, THREADS, FAM>, THREADS,
                                                     smem) != cudaSuccess || fit < 1)
@@ -1788,11 +1796,11 @@ cudaError_t persist_any(int fam, const Ctx& c, const Item* items, int nitems, in
 }
 
 // resident CTAs per SM of `kernel` with its stage requested or not
-template <int FAM, int THREADS, typename K>
+template <typename T, int FAM, int THREADS, typename K>
 int fit_of(K kernel, int stage) {
-  const int smem = stage_smem<FAM, THREADS>(kernel, stage);
-  int n = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, THREADS, smem) != cudaSuccess)
+  int smem = 0, n = 0;
+  if (stage_smem<T, FAM, THREADS>(kernel, stage, smem) != cudaSuccess ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, THREADS, smem) != cudaSuccess)
     return 1;
   return n > 0 ? n : 1;
 }
@@ -1800,10 +1808,10 @@ int fit_of(K kernel, int stage) {
 template <typename T, int FAM>
 int persist_fit_fam(int threads, int st) {
   switch (threads) {
-    case 64: return fit_of<FAM, 64>(k_persist<T, 64, FAM>, st);
-    case 128: return fit_of<FAM, 128>(k_persist<T, 128, FAM>, st);
-    case 512: return fit_of<FAM, 512>(k_persist<T, 512, FAM>, st);
-    default: return fit_of<FAM, 256>(k_persist<T, 256, FAM>, st);
+    case 64: return fit_of<T, FAM, 64>(k_persist<T, 64, FAM>, st);
+    case 128: return fit_of<T, FAM, 128>(k_persist<T, 128, FAM>, st);
+    case 512: return fit_of<T, FAM, 512>(k_persist<T, 512, FAM>, st);
+    default: return fit_of<T, FAM, 256>(k_persist<T, 256, FAM>, st);
   }
 }
 
@@ -1833,11 +1841,11 @@ cudaError_t launch_fam(const Ctx& c, const Item* items, int nitems, int threads,
 template <typename T, int FAM>
 int resident_fam(int threads, int st) {
   switch (threads) {
-    case 32: return fit_of<FAM, 32>(k_stream<T, 32, FAM>, st);
-    case 64: return fit_of<FAM, 64>(k_stream<T, 64, FAM>, st);
-    case 128: return fit_of<FAM, 128>(k_stream<T, 128, FAM>, st);
-    case 512: return fit_of<FAM, 512>(k_stream<T, 512, FAM>, st);
-    default: return fit_of<FAM, 256>(k_stream<T, 256, FAM>, st);
+    case 32: return fit_of<T, FAM, 32>(k_stream<T, 32, FAM>, st);
+    case 64: return fit_of<T, FAM, 64>(k_stream<T, 64, FAM>, st);
+    case 128: return fit_of<T, FAM, 128>(k_stream<T, 128, FAM>, st);
+    case 512: return fit_of<T, FAM, 512>(k_stream<T, 512, FAM>, st);
+    default: return fit_of<T, FAM, 256>(k_stream<T, 256, FAM>, st);
   }
 }
 
