@@ -196,9 +196,10 @@ typedef struct bc_grid {
  *              is one application of A: every row reads the input values, so
  *              Sync rows are computed into a plan-owned staging buffer and
  *              written after all other rows have read the data (when all of
- *              them fall into groups of at most four that read exactly the
- *              cells they write, each group is summed and stored in place
- *              after those rows instead).  Two Sync
+ *              them fall into groups of at most four rows, of at most four
+ *              entries each, that read only the cells the group writes, each
+ *              group is summed and stored in place after those rows
+ *              instead).  Two Sync
  *              boxes must not share a data cell (BC_ERR_OVERLAP).  Because of
  *              the staging buffer, applies of one plan with Sync rows must
  *              not run concurrently on several streams.

@@ -320,9 +320,16 @@ struct SyncCtx {
   int level_fast = 0;   // 1: consecutive threads take consecutive levels
                         //    (levels contiguous in memory), 0: consecutive
                         //    rows at one level
-  // closed groups of rows (ngroups 0: none): up to four rows, -1 past the last
+  // closed groups of up to kSyncGroup rows of up to kSyncGroup entries that
+  // read only the cells the group writes (ngroups 0: none).  Four planes of
+  // ngroups int4: the rows' slots, data offsets (level 0), level strides (a
+  // row past the last repeats the first) and {columns of rows 0 and 1, of rows
+  // 2 and 3, levels, rows}; a row's columns take 16 bits: its entry count, then
+  // two bits per entry (the row whose cell it reads) in entry order.  group_w:
+  // kSyncGroup planes of ngroups x kSyncGroup weights, a row's in entry order.
   int ngroups = 0;
   const int4* group = nullptr;
+  const void* group_w = nullptr;
   const int4* row = nullptr;
   const int32_t* ptr = nullptr;
   const int2* ent = nullptr;
@@ -333,6 +340,7 @@ struct SyncCtx {
   const void* cw = nullptr;
   void* stage = nullptr;
 };
+constexpr int kSyncGroup = 4;
 enum SyncStep : int32_t {
   SYNC_ROWS = 0,      // stage = A_sync x (reads data)
   SYNC_COMMIT = 1,    // data = stage

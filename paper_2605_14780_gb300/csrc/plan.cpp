@@ -189,7 +189,10 @@ struct bc_plan {
     std::vector<int32_t> cstage;
     std::vector<double> cw;
     int64_t stage = 0;  // staging values (rows x levels)
-    std::vector<int4> group;  // closed groups of rows, when all rows are in one
+    // closed groups of rows (the rows, -1 past the last), when all rows are in
+    // one; their records and weights (SyncCtx::group, group_w)
+    std::vector<int4> group, grec;
+    std::vector<double> gw;
   } sync;
   SyncCtx sync_ctx{};
   // work lists
@@ -606,8 +609,9 @@ bc_status add_sync(bc_plan* P, const bc_submatrix& m, int idx, Coverage& dcov) {
   return BC_OK;
 }
 
-// Groups of at most four Sync rows that read exactly the cells they write;
-// none when some row is in no such group.
+// Groups of at most kSyncGroup Sync rows of at most kSyncGroup entries that
+// read exactly the cells they write, and their records; none when some row is
+// in no such group.
 void build_sync_groups(bc_plan* P) {
   auto& S = P->sync;
   S.group.clear();
@@ -620,15 +624,19 @@ void build_sync_groups(bc_plan* P) {
     while (up[r] != r) r = up[r] = up[up[r]];
     return r;
   };
-  for (size_t r = 0; r < n; ++r)
+  std::vector<int32_t> col(S.ent.size());  // the row whose cell an entry reads
+  for (size_t r = 0; r < n; ++r) {
+    if (S.ptr[r + 1] - S.ptr[r] > kSyncGroup) return;
     for (int32_t e = S.ptr[r]; e < S.ptr[r + 1]; ++e) {
       const auto it = row_of.find(col_key(S.ent[e].x, S.ent[e].y));
       if (it == row_of.end()) return;  // reads a cell that no row writes
+      col[e] = it->second;
       const int32_t a = root((int32_t)r), b = root(it->second);
       if (a != b) up[std::max(a, b)] = std::min(a, b);
     }
+  }
   // groups in the order of their first rows, rows ascending
-  std::vector<int32_t> group_of(n, -1);
+  std::vector<int32_t> group_of(n, -1), place(n, 0);
   std::vector<int4> groups;
   for (size_t r = 0; r < n; ++r) {
     int32_t& g = group_of[root((int32_t)r)];
@@ -637,15 +645,43 @@ void build_sync_groups(bc_plan* P) {
       groups.push_back(make_int4((int)r, -1, -1, -1));
     } else if (groups[g].y < 0) {
       groups[g].y = (int)r;
+      place[r] = 1;
     } else if (groups[g].z < 0) {
       groups[g].z = (int)r;
+      place[r] = 2;
     } else if (groups[g].w < 0) {
       groups[g].w = (int)r;
+      place[r] = 3;
     } else {
       return;
     }
   }
   S.group.swap(groups);
+  const size_t ng = S.group.size();
+  S.grec.assign(4 * ng, make_int4(0, 0, 0, 0));
+  S.gw.assign(kSyncGroup * ng * kSyncGroup, 0.0);
+  for (size_t g = 0; g < ng; ++g) {
+    const int rows[kSyncGroup] = {S.group[g].x, S.group[g].y, S.group[g].z, S.group[g].w};
+    int slot[kSyncGroup], off[kSyncGroup], ls[kSyncGroup], bits[kSyncGroup] = {0, 0, 0, 0}, nr = 0;
+    for (int k = 0; k < kSyncGroup; ++k) {
+      const int r = rows[k] < 0 ? rows[0] : rows[k];
+      slot[k] = S.row[r].x;
+      off[k] = S.row[r].y;
+      ls[k] = P->slot_ls[slot[k]];
+      if (rows[k] < 0) continue;
+      ++nr;
+      bits[k] = S.ptr[r + 1] - S.ptr[r];
+      for (int32_t e = S.ptr[r]; e < S.ptr[r + 1]; ++e) {
+        bits[k] |= place[col[e]] << (3 + 2 * (e - S.ptr[r]));
+        S.gw[(k * ng + g) * kSyncGroup + (e - S.ptr[r])] = S.w[e];
+      }
+    }
+    S.grec[g] = make_int4(slot[0], slot[1], slot[2], slot[3]);
+    S.grec[ng + g] = make_int4(off[0], off[1], off[2], off[3]);
+    S.grec[2 * ng + g] = make_int4(ls[0], ls[1], ls[2], ls[3]);
+    S.grec[3 * ng + g] = make_int4(bits[0] | bits[1] << 16, bits[2] | bits[3] << 16,
+                                   S.row[rows[0]].w, nr);
+  }
 }
 
 // Columns read by Sync rows and their entries {staging offset, weight}, in
@@ -1906,7 +1942,8 @@ bc_status upload_tables(bc_plan* P) {
   const size_t o_ew = L.take(P->aent_w.size() * S);
   const auto& Y = P->sync;
   const size_t o_yr = L.take(Y.row.size() * sizeof(int4));
-  const size_t o_yg = L.take(Y.group.size() * sizeof(int4));
+  const size_t o_yg = L.take(Y.grec.size() * sizeof(int4));
+  const size_t o_ygw = L.take(Y.gw.size() * S);
   const size_t o_yp = L.take(Y.ptr.size() * 4);
   const size_t o_ye = L.take(Y.ent.size() * sizeof(int2));
   const size_t o_yw = L.take(Y.w.size() * S);
@@ -1918,7 +1955,7 @@ bc_status upload_tables(bc_plan* P) {
   const size_t o_ctr = L.take(kCtrWords * kFamilies * kCounterStreams * sizeof(unsigned));  // zero
   std::vector<char> host(L.off + 256, 0);
   put_raw(host, o_yr, Y.row);
-  put_raw(host, o_yg, Y.group);
+  put_raw(host, o_yg, Y.grec);
   put_raw(host, o_yp, Y.ptr);
   put_raw(host, o_ye, Y.ent);
   put_raw(host, o_yc, Y.col);
@@ -1945,6 +1982,7 @@ bc_status upload_tables(bc_plan* P) {
     put_dtype<double>(host, o_k, P->const_val);
     put_dtype<double>(host, o_ew, P->aent_w);
     put_dtype<double>(host, o_yw, Y.w);
+    put_dtype<double>(host, o_ygw, Y.gw);
     put_dtype<double>(host, o_ycw, Y.cw);
   } else {
     put_dtype<float>(host, o_w, P->itp_w);
@@ -1954,6 +1992,7 @@ bc_status upload_tables(bc_plan* P) {
     put_dtype<float>(host, o_k, P->const_val);
     put_dtype<float>(host, o_ew, P->aent_w);
     put_dtype<float>(host, o_yw, Y.w);
+    put_dtype<float>(host, o_ygw, Y.gw);
     put_dtype<float>(host, o_ycw, Y.cw);
   }
   cudaError_t e = dev_malloc(&P->tables.base, host.size());
@@ -1997,6 +2036,7 @@ bc_status upload_tables(bc_plan* P) {
   y.row = reinterpret_cast<const int4*>(b + o_yr);
   y.ngroups = (int)Y.group.size();
   y.group = reinterpret_cast<const int4*>(b + o_yg);
+  y.group_w = b + o_ygw;
   y.ptr = reinterpret_cast<const int32_t*>(b + o_yp);
   y.ent = reinterpret_cast<const int2*>(b + o_ye);
   y.w = b + o_yw;
@@ -3778,20 +3818,32 @@ int64_t check_sync(WorkCheck& W) {
     for (int32_t e = Y.ptr[u]; e < Y.ptr[u + 1]; ++e)
       want[col_key(Y.ent[(size_t)e].x, Y.ent[(size_t)e].y)].push_back({r.z, Y.w[(size_t)e]});
   }
-  // closed groups: every row in one group, reading only cells its group writes
+  // closed groups: every row in one group, whose record gives its cell and its
+  // entries in order
   std::vector<int> grouped(Y.row.size(), 0);
-  for (const int4& g : Y.group) {
-    const int rows[4] = {g.x, g.y, g.z, g.w};
-    std::unordered_set<int64_t> cells;
-    for (int r : rows)
-      if (r >= 0) {
-        ++grouped[(size_t)r];
-        cells.insert(col_key(Y.row[(size_t)r].x, Y.row[(size_t)r].y));
+  const size_t ng = Y.group.size();
+  for (size_t g = 0; g < ng; ++g) {
+    const int rows[kSyncGroup] = {Y.group[g].x, Y.group[g].y, Y.group[g].z, Y.group[g].w};
+    const int4 sl = Y.grec[g], of = Y.grec[ng + g], st = Y.grec[2 * ng + g], me = Y.grec[3 * ng + g];
+    const int slot[kSyncGroup] = {sl.x, sl.y, sl.z, sl.w}, off[kSyncGroup] = {of.x, of.y, of.z, of.w};
+    const int ls[kSyncGroup] = {st.x, st.y, st.z, st.w};
+    const int col[kSyncGroup] = {me.x & 0xffff, (int)((unsigned)me.x >> 16), me.y & 0xffff,
+                                 (int)((unsigned)me.y >> 16)};
+    for (int k = 0; k < kSyncGroup; ++k) {
+      const int r = rows[k];
+      if ((r >= 0) != (k < me.w)) W.problem("a Sync group counts its rows wrongly", sl.x, of.x);
+      if (r < 0) continue;
+      ++grouped[(size_t)r];
+      const int4 row = Y.row[(size_t)r];
+      bool ok = slot[k] == row.x && off[k] == row.y && me.z == row.w &&
+                ls[k] == W.ls_of_slot(row.x) && (col[k] & 7) == Y.ptr[r + 1] - Y.ptr[r];
+      for (int32_t e = Y.ptr[r]; ok && e < Y.ptr[r + 1]; ++e) {
+        const int c = col[k] >> (3 + 2 * (e - Y.ptr[r])) & 3;
+        ok = c < me.w && slot[c] == Y.ent[e].x && off[c] == Y.ent[e].y &&
+             Y.gw[(k * ng + g) * kSyncGroup + (e - Y.ptr[r])] == Y.w[e];
       }
-    for (int r : rows)
-      for (int32_t e = r >= 0 ? Y.ptr[(size_t)r] : 0; r >= 0 && e < Y.ptr[(size_t)r + 1]; ++e)
-        if (!cells.count(col_key(Y.ent[(size_t)e].x, Y.ent[(size_t)e].y)))
-          W.problem("a Sync group reads a cell it does not write", Y.row[(size_t)r].x, Y.row[(size_t)r].y);
+      if (!ok) W.problem("a Sync group's record differs from its row", row.x, row.y);
+    }
   }
   for (size_t r = 0; !Y.group.empty() && r < grouped.size(); ++r)
     if (grouped[r] != 1) W.problem("a Sync row is not in one group", Y.row[r].x, Y.row[r].y);

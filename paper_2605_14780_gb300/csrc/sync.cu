@@ -81,63 +81,81 @@ __global__ void __launch_bounds__(kSyncThreads) k_sync(SyncCtx s, int step, void
 }
 
 // Closed groups: up to four rows that read exactly the cells they write (the
-// copies of one node), so one thread sums them all and then stores them, with
-// no staging: the cells' DRAM granules (a node of a column is 4 bytes of 64)
-// are read and written once, in one launch instead of two, and the rows'
-// tables load once for LV levels.  Runs after every kernel that reads data.
-// Shared nodes of 8 x 8 blocks of 129^2 x 96 planes FP32: 41 us for the rows
-// beside the ghost kernel and 41 for the commit -> 46 us, the whole fill 132 ->
-// 110 us.
-constexpr int kSyncLevels = 4;  // levels of a thread where they are far apart
+// copies of one node), so one thread sums them all at one level and then
+// stores them, with no staging: the cells' DRAM granules (a node of a column is
+// 4 bytes of 64) are read and written once, in one launch instead of two.  Runs
+// after every kernel that reads data.  Bound by DRAM granules on large grids
+// and by its chain of dependent loads on small ones, so a group comes as a
+// record (SyncCtx::group): record, slot pointers, values is the whole chain,
+// each distinct cell is loaded once, and the rows are summed from registers in
+// entry order.  One level a thread and CTAs of 64 threads spread a small grid
+// over the SMs (four levels a thread, which saves table loads: within 2 % on
+// large grids, 30 % slower on small FP64 ones, whose multiply-adds then queue on
+// a few SMs).
+// 8 x 8 blocks of 129^2 x 96 planes FP32, the whole fill: 133 us staged, 99 with
+// the rows' own tables walked in series, 90 so; 2 x 2 blocks of 9^2 x 2 planes
+// FP64: 5.8, 9.3, 5.3 us.
+constexpr int kGroupThreads = 64;
 
-template <typename T, int LV>
-__global__ void __launch_bounds__(kSyncThreads)
-    k_sync_groups(SyncCtx s, void* const* slots, const int32_t* slot_ls) {
-  const int64_t t = (int64_t)blockIdx.x * kSyncThreads + threadIdx.x;
-  int u, l0;
-  if (LV == 1) {  // levels contiguous: levels fastest
-    u = (int)(t / s.lmax);
-    l0 = (int)(t - (int64_t)u * s.lmax);
+template <typename T>
+__device__ __forceinline__ void load_row_weights(const T* p, T (&w)[kSyncGroup]) {
+  if constexpr (sizeof(T) == 4) {
+    const float4 v = __ldg(reinterpret_cast<const float4*>(p));
+    w[0] = v.x;
+    w[1] = v.y;
+    w[2] = v.z;
+    w[3] = v.w;
   } else {
-    const int64_t c = t / s.ngroups;
-    u = (int)(t - c * s.ngroups);
-    l0 = (int)c * LV;
+    const double2 v = __ldg(reinterpret_cast<const double2*>(p));
+    const double2 u = __ldg(reinterpret_cast<const double2*>(p) + 1);
+    w[0] = v.x;
+    w[1] = v.y;
+    w[2] = u.x;
+    w[3] = u.y;
   }
-  if (u >= s.ngroups || l0 >= s.lmax) return;
-  const int4 g = __ldg(s.group + u);
-  const int rows[4] = {g.x, g.y, g.z, g.w};
-  T acc[4][LV];
-  T* d[4];
-  int64_t dls[4];
-  int nl = 0;
+}
+
+template <typename T>
+__global__ void __launch_bounds__(kGroupThreads) k_sync_groups(SyncCtx s, void* const* slots) {
+  const int64_t t = (int64_t)blockIdx.x * kGroupThreads + threadIdx.x;
+  if (t >= (int64_t)s.ngroups * s.lmax) return;
+  int u, l;
+  split(s, s.ngroups, t, u, l);
+  const int64_t ng = s.ngroups;
+  const int4 sl = __ldg(s.group + u), of = __ldg(s.group + ng + u), st = __ldg(s.group + 2 * ng + u),
+             me = __ldg(s.group + 3 * ng + u);
+  const int slot[kSyncGroup] = {sl.x, sl.y, sl.z, sl.w}, off[kSyncGroup] = {of.x, of.y, of.z, of.w};
+  const int ls[kSyncGroup] = {st.x, st.y, st.z, st.w};
+  const int col[kSyncGroup] = {me.x & 0xffff, (int)((unsigned)me.x >> 16), me.y & 0xffff,
+                               (int)((unsigned)me.y >> 16)};
+  const int nr = me.w;
+  if (l >= me.z) return;
+  T* d[kSyncGroup];
 #pragma unroll
-  for (int r = 0; r < 4; ++r) {
+  for (int r = 0; r < kSyncGroup; ++r)
+    d[r] = slot_at<T>(slots, slot[r], off[r]) + (int64_t)l * ls[r];
+  T x[kSyncGroup], w[kSyncGroup][kSyncGroup];
 #pragma unroll
-    for (int l = 0; l < LV; ++l) acc[r][l] = T(0);
-    if (rows[r] < 0) continue;
-    const int4 rw = __ldg(s.row + rows[r]);
-    nl = rw.w - l0;
-    if (nl <= 0) return;  // a group's rows have one level count
-    dls[r] = __ldg(slot_ls + rw.x);
-    d[r] = slot_at<T>(slots, rw.x, rw.y) + l0 * dls[r];
-    const int e0 = __ldg(s.ptr + rows[r]), e1 = __ldg(s.ptr + rows[r] + 1);
-    for (int e = e0; e < e1; ++e) {
-      const int2 en = __ldg(s.ent + e);
-      const T w = __ldg(static_cast<const T*>(s.w) + e);
-      const int64_t xls = __ldg(slot_ls + en.x);
-      const T* x = slot_at<T>(slots, en.x, en.y) + l0 * xls;
-#pragma unroll
-      for (int l = 0; l < LV; ++l)
-        if (l < nl) acc[r][l] = fma(w, x[l * xls], acc[r][l]);
-    }
+  for (int r = 0; r < kSyncGroup; ++r) {
+    x[r] = T(0);
+    if (r >= nr) continue;  // no entry reads it
+    load_row_weights<T>(static_cast<const T*>(s.group_w) + (r * ng + u) * kSyncGroup, w[r]);
+    x[r] = *d[r];
   }
 #pragma unroll
-  for (int r = 0; r < 4; ++r)
-    if (rows[r] >= 0) {
+  for (int r = 0; r < kSyncGroup; ++r) {
+    if (r >= nr) continue;
+    T acc = T(0);
+    const int n = col[r] & 7;
 #pragma unroll
-      for (int l = 0; l < LV; ++l)
-        if (l < nl) d[r][l * dls[r]] = acc[r][l];
-    }
+    for (int e = 0; e < kSyncGroup; ++e)
+      if (e < n) {
+        const int c = col[r] >> (3 + 2 * e);
+        const T lo = c & 1 ? x[1] : x[0], hi = c & 1 ? x[3] : x[2];
+        acc = fma(w[r][e], c & 2 ? hi : lo, acc);
+      }
+    *d[r] = acc;
+  }
 }
 
 }  // namespace
@@ -146,11 +164,10 @@ cudaError_t launch_sync(int dtype, int step, const SyncCtx& s, void* const* slot
                         const int32_t* slot_ls, cudaStream_t stream) {
   if (step == SYNC_GROUPS) {
     if (s.ngroups <= 0) return cudaSuccess;
-    const int64_t parts = s.level_fast ? s.lmax : (s.lmax + kSyncLevels - 1) / kSyncLevels;
-    const int blocks = (int)((s.ngroups * parts + kSyncThreads - 1) / kSyncThreads);
-    auto* k = dtype == 1 ? (s.level_fast ? k_sync_groups<double, 1> : k_sync_groups<double, kSyncLevels>)
-                         : (s.level_fast ? k_sync_groups<float, 1> : k_sync_groups<float, kSyncLevels>);
-    k<<<blocks, kSyncThreads, 0, stream>>>(s, slots, slot_ls);
+    const int64_t n = (int64_t)s.ngroups * s.lmax;
+    const int blocks = (int)((n + kGroupThreads - 1) / kGroupThreads);
+    auto* k = dtype == 1 ? k_sync_groups<double> : k_sync_groups<float>;
+    k<<<blocks, kGroupThreads, 0, stream>>>(s, slots);
     return cudaGetLastError();
   }
   const int64_t n = (int64_t)(step == SYNC_ADJOINT ? s.ncols : s.nrows) * s.lmax;
