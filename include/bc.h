@@ -290,9 +290,9 @@ typedef struct bc_plan_opts {
   int32_t level_chunk;     /* levels one lane carries through a table row
                               when levels are far apart in memory
                               (interpolation, CSR and transpose rows): 0
-                              default (4 for interpolation and transpose
-                              rows, 8 for CSR rows; staged tiles as many as
-                              they hold), or 1, 2, 4, 8 for all;
+                              default (4, but 2 for vector pairs and 8 for
+                              FP32 CSR rows; staged tiles as many as they
+                              hold), or 1, 2, 4, 8 for all;
                               the launches of every kind in one kernel
                               (BC_BATCH_PERSISTENT, BC_BATCH_SINGLE) take
                               at most 4                                     */

@@ -941,14 +941,24 @@ int table_mode(const bc_block& B, int order, int chunk) {
   return std::min(B.nlevels, chunk);
 }
 
-// levels per unit of the chunked unit order (bc_plan_opts.level_chunk; by
-// default 4 for interpolation rows, whose pair path keeps two components'
-// sums, and for transpose rows, whose longest chain ends the launch
-// (the 6 x 768^2 adjoint 107 us at 8, 79 us at 4), and 8 for CSR rows); the persistent launch's kernel holds at
-// most 4
-int level_chunk(const bc_plan* P, int fam) {
+// Levels per unit of the chunked unit order (bc_plan_opts.level_chunk), by
+// default
+//  - 4 for interpolation rows, 2 for vector pairs, which keep two components'
+//    sums (6 x 512 rows of scattered 4-point nodes, (h, u, v) x 32 levels: FP32
+//    5.4 us at 4, 4.3 at 2, FP64 7.3 and 5.5; eight times the rows: FP32 22 and
+//    22, FP64 32 and 32);
+//  - 4 for transpose rows, whose longest chain ends the launch (the 6 x 768^2
+//    adjoint 107 us at 8, 79 us at 4);
+//  - for CSR rows 8 in FP32 and 4 in FP64, where 8 levels' sums spill (12 288
+//    rows of 16 entries x 32 levels: 36 us at 8, 20 at 4 with two rows to a
+//    patch, 19 and 18 with full reuse; 512 blocks: 154 and 140).
+// The kernel of all kinds holds at most 4.
+int level_chunk(const bc_plan* P, int kind) {
   int ch = P->opts.level_chunk;
-  if (ch == 0) ch = fam == FAM_CSR ? 8 : 4;
+  if (ch == 0) {
+    ch = kind == IK_INTERP_PAIR ? 2 : 4;
+    if (kind == IK_CSR && P->dtype == BC_F32) ch = 8;
+  }
   const bool all_kinds =
       P->opts.batch_mode == BC_BATCH_PERSISTENT || P->opts.batch_mode == BC_BATCH_SINGLE;
   return all_kinds ? std::min(ch, 4) : ch;
@@ -1430,11 +1440,7 @@ void build_items(bc_plan* P) {
     }
   }
   auto table_emit = [&](std::vector<Item>& out, const Item& it, const bc_block& B, int vol) {
-    const bool interp = it.kind == IK_INTERP || it.kind == IK_INTERP_PAIR;
-    int mode = table_mode(B, P->opts.unit_order,
-                                it.kind == IK_CSR ? level_chunk(P, FAM_CSR)
-                                : interp          ? level_chunk(P, FAM_INTERP)
-                                                  : level_chunk(P, FAM_ADJ));
+    int mode = table_mode(B, P->opts.unit_order, level_chunk(P, it.kind));
     if (mode == MODE_FLAT_LEVEL) mode = MODE_SPLIT;
     const int flat_item =
         mode == MODE_SPLIT ? std::max(32, per_table_flat_item / kLevelSplit / 32 * 32) : per_table_flat_item;
@@ -1481,7 +1487,7 @@ void build_items(bc_plan* P) {
           }
           // levels far apart in memory: stage the nodes of each tile in
           // shared memory when the tiles' boxes are small
-          const int mode = table_mode(B, P->opts.unit_order, level_chunk(P, FAM_INTERP));
+          const int mode = table_mode(B, P->opts.unit_order, level_chunk(P, it.kind));
           if (mode < 2 || P->opts.unstaged_rows ||
               !emit_tiles(P, s, it, out))
             table_emit(out, it, B, s.vol);
@@ -1498,7 +1504,7 @@ void build_items(bc_plan* P) {
             it.src_ls = (int32_t)(S.nlevels > 1 ? S.level_stride : 0);
           }
           // levels far apart in memory: stage each tile's column box
-          const int mode = table_mode(B, P->opts.unit_order, level_chunk(P, FAM_CSR));
+          const int mode = table_mode(B, P->opts.unit_order, level_chunk(P, it.kind));
           if (mode < 2 || P->opts.unstaged_rows ||
               !emit_csr_tiles(P, s, (int)ci, it, out))
             table_emit(out, it, B, s.vol);
@@ -1653,7 +1659,7 @@ void build_items(bc_plan* P) {
       it.src_ls = (int32_t)(G.nlevels > 1 ? G.level_stride : 0);
     }
     // levels far apart in memory: stage each tile's box of ghost cotangents
-    const int mode = table_mode(B0, P->opts.unit_order, level_chunk(P, FAM_ADJ));
+    const int mode = table_mode(B0, P->opts.unit_order, level_chunk(P, it.kind));
     if (mode < 2 || P->opts.unstaged_rows ||
         !emit_adj_tiles(P, r0, r1 - r0, it, mode, B0.nlevels, P->adj_items))
       table_emit(P->adj_items, it, B0, r1 - r0);
