@@ -1156,12 +1156,39 @@ void push_tile(const bc_plan* P, const TileBox& T, int q0, int nq, const Item& p
   }
 }
 
+// The staged tiles of one kind of rows over a plan: their rows, the entries
+// these read and the box cells that hold them.
+struct TileSums {
+  int64_t tiles = 0, rows = 0, entries = 0, cells = 0;
+};
+
+// Plans of at most this many values an SM take FP64 tiles half full (below).
+constexpr int64_t kSmallTilePlan = 640;
+
+// Whether interpolation tiles beat the per-lane rows.  A tile costs a warp
+// however few rows fill it, so nodes that lie apart (scattered, or a source
+// block that runs askew or is finer) cut tiles that lose.  FP32: six rows a
+// tile on average (6 x 384^2, (h, u, v) x 32 levels, 4-point rows in groups
+// that share a strip: 3 rows 72 us staged, 54 per lane; 5: 54, 51; 6: 48.7,
+// 48.7; 8: 43, 48; 32: 14.6, 17.4).  FP64 multiply-adds fill their pipe (29 us
+// of it there), which idle lanes waste: 24 rows (8: 108 and 60 us; 16: 66 and
+// 58), each staged value read three times (twice, 31 rows: 38 and 30; 3.7
+// times, 32 rows: 30 and 29; 6-point rows of 6 x 600^2: 64.6 and 67.5).  In
+// small plans latency counts instead: 16 rows (6 x 33^2 x 32 levels, tiles of
+// 32 and 1 rows: 4.8 and 6.8 us).
+bool keep_interp_tiles(const bc_plan* P, const TileSums& n, int64_t plan_values) {
+  if (P->dtype == BC_F32) return n.rows >= 6 * n.tiles;
+  const bool small = plan_values <= kSmallTilePlan * std::max(1, P->num_sms);
+  return n.rows >= (small ? 16 : 24) * n.tiles && n.entries >= 3 * n.cells;
+}
+
 // Staged interpolation items of sub-matrix s: tiles of up to kTileCells
 // consecutive box cells, each as long as its cells' nodes lie in one 2-D
 // source block inside a box of one plane (kPlaneInterp cells).  Writes the
-// cells' itp_box rows.  Returns false (the sub-matrix keeps the per-lane
-// path) when some cell does not qualify.
-bool emit_tiles(bc_plan* P, const Sub& s, const Item& proto, std::vector<Item>& out) {
+// cells' itp_box rows and adds to `sums`.  Returns false (the sub-matrix keeps
+// the per-lane path) when some cell does not qualify.
+bool emit_tiles(bc_plan* P, const Sub& s, const Item& proto, std::vector<Item>& out,
+                TileSums& sums) {
   const int L = P->blocks[s.block].nlevels;
   std::vector<Item> tiles;
   std::vector<std::pair<int, int32_t>> boxes;  // (row, itp_box) to write on success
@@ -1169,6 +1196,7 @@ bool emit_tiles(bc_plan* P, const Sub& s, const Item& proto, std::vector<Item>& 
     int i, j, rows, snap;
   };
   std::vector<Node0> n0;
+  TileSums mine;
   for (int q0 = 0; q0 < s.vol;) {
     int base = -1;
     TileBox T;
@@ -1195,6 +1223,7 @@ bool emit_tiles(bc_plan* P, const Sub& s, const Item& proto, std::vector<Item>& 
       T = G;
       base = ix.x;
       n0.push_back({i, j, ax, snap ? 1 : 0});
+      mine.entries += np;
     }
     const int nq = (int)n0.size();
     if (nq == 0) return false;
@@ -1207,7 +1236,14 @@ bool emit_tiles(bc_plan* P, const Sub& s, const Item& proto, std::vector<Item>& 
                                              (n0[q].snap ? kBoxSnap : 0)});
     push_tile(P, T, q0, nq, proto, L, tiles);
     q0 += nq;
+    ++mine.tiles;
+    mine.rows += nq;
+    mine.cells += T.cells();
   }
+  sums.tiles += mine.tiles;
+  sums.rows += mine.rows;
+  sums.entries += mine.entries;
+  sums.cells += mine.cells;
   for (const auto& b : boxes) P->itp_box[(size_t)b.first] = b.second;
   out.insert(out.end(), tiles.begin(), tiles.end());
   return true;
@@ -1447,6 +1483,12 @@ void build_items(bc_plan* P) {
     emit_units(out, it, vol, B.nlevels, mode, mode < 2 ? flat_item : per_table_item);
   };
   std::vector<std::pair<int, std::vector<Item>>> per_sub(P->subs.size());
+  // rows with levels far apart in memory, staged below if that pays
+  struct Rows {
+    size_t sub;
+    Item proto;
+  };
+  std::vector<Rows> interp_rows;
   for (size_t si = 0; si < P->subs.size(); ++si) {
     const Sub& s = P->subs[si];
     const bc_block& B = P->blocks[s.block];
@@ -1485,12 +1527,11 @@ void build_items(bc_plan* P) {
           } else {
             it.kind = IK_INTERP;
           }
-          // levels far apart in memory: stage the nodes of each tile in
-          // shared memory when the tiles' boxes are small
           const int mode = table_mode(B, P->opts.unit_order, level_chunk(P, it.kind));
-          if (mode < 2 || P->opts.unstaged_rows ||
-              !emit_tiles(P, s, it, out))
+          if (mode < 2 || P->opts.unstaged_rows)
             table_emit(out, it, B, s.vol);
+          else
+            interp_rows.push_back({si, it});
           break;
         }
         case BC_CSR: {
@@ -1513,6 +1554,31 @@ void build_items(bc_plan* P) {
       }
     }
   }
+  // The rows of a kind are staged in the whole plan or nowhere: the shared
+  // memory of a few tiles would cost the per-lane items beside them occupancy.
+  auto per_lane = [&](const Rows& r) {
+    const Sub& s = P->subs[r.sub];
+    table_emit(per_sub[r.sub].second, r.proto, P->blocks[s.block], s.vol);
+  };
+  auto stage_rows = [&](const std::vector<Rows>& rows, auto emit, auto keep) {
+    TileSums sums;
+    std::vector<std::vector<Item>> tiles(rows.size());
+    for (size_t k = 0; k < rows.size(); ++k)
+      if (!emit(rows[k], tiles[k], sums)) tiles[k].clear();
+    const bool staged = sums.tiles > 0 && keep(P, sums, total_values);
+    for (size_t k = 0; k < rows.size(); ++k) {
+      std::vector<Item>& out = per_sub[rows[k].sub].second;
+      if (staged && !tiles[k].empty())
+        out.insert(out.end(), tiles[k].begin(), tiles[k].end());
+      else
+        per_lane(rows[k]);
+    }
+  };
+  stage_rows(interp_rows,
+             [&](const Rows& r, std::vector<Item>& out, TileSums& sums) {
+               return emit_tiles(P, P->subs[r.sub], r.proto, out, sums);
+             },
+             keep_interp_tiles);
   // order: by kind, then sub-matrix (per-sub and per-kind ranges contiguous)
   P->items.clear();
   P->sub_begin.assign(P->subs.size(), 0);
