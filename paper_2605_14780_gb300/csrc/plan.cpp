@@ -1160,6 +1160,12 @@ void push_tile(const bc_plan* P, const TileBox& T, int q0, int nq, const Item& p
 // these read and the box cells that hold them.
 struct TileSums {
   int64_t tiles = 0, rows = 0, entries = 0, cells = 0;
+  void operator+=(const TileSums& o) {
+    tiles += o.tiles;
+    rows += o.rows;
+    entries += o.entries;
+    cells += o.cells;
+  }
 };
 
 // Plans of at most this many values an SM take FP64 tiles half full (below).
@@ -1236,23 +1242,33 @@ bool emit_tiles(bc_plan* P, const Sub& s, const Item& proto, std::vector<Item>& 
                                              (n0[q].snap ? kBoxSnap : 0)});
     push_tile(P, T, q0, nq, proto, L, tiles);
     q0 += nq;
-    ++mine.tiles;
-    mine.rows += nq;
-    mine.cells += T.cells();
+    mine += {1, nq, 0, T.cells()};
   }
-  sums.tiles += mine.tiles;
-  sums.rows += mine.rows;
-  sums.entries += mine.entries;
-  sums.cells += mine.cells;
+  sums += mine;
   for (const auto& b : boxes) P->itp_box[(size_t)b.first] = b.second;
   out.insert(out.end(), tiles.begin(), tiles.end());
   return true;
 }
 
-// Staging pays only when a tile's entries read each staged value at least
-// this often on average (a box mostly of values no row reads costs more
-// loads than it saves).
+// Staging pays only when the entries read each staged value at least this
+// often on average (a box mostly of values no row reads costs more loads than
+// it saves).
 constexpr double kMinTileReuse = 1.5;
+
+// Whether CSR tiles beat the per-lane rows (the comparison of
+// keep_interp_tiles; a tile that happens to be short, such as the last row of a
+// strip, does not decide for its neighbours: reconstruction rows of 6 x 33^2,
+// (h, u, v) x 32 levels FP32, 23.5 us with such components per lane, 6.9 so).
+// FP32: twelve rows a tile on average (6 x 384^2, 16-entry rows x 32 levels in
+// groups that share a patch: 8 rows 13.4 us staged, 11.9 per lane; 12: 11.7,
+// 11.4; 14: 10.9, 11.7; 20: 8.3, 11.0).  FP64, whose pipe idle lanes waste: 28
+// rows (16: 39 and 24 us; 28: 24.9 and 23.6; 32: 22.5 and 23.4), or 16 in small
+// plans.
+bool keep_csr_tiles(const bc_plan* P, const TileSums& n, int64_t plan_values) {
+  const bool small = plan_values <= kSmallTilePlan * std::max(1, P->num_sms);
+  const int least = P->dtype == BC_F32 ? 12 : (small ? 16 : 28);
+  return n.rows >= least * n.tiles && (double)n.entries >= kMinTileReuse * (double)n.cells;
+}
 
 // Staged tiles of rows [q, q1) (`entries(q, f)` calls f(slot, offset,
 // weight) for each entry of row q in order): the longest tile of at most
@@ -1265,6 +1281,7 @@ constexpr double kMinTileReuse = 1.5;
 struct TileEntries {
   std::vector<int32_t> box;
   std::vector<double> w;
+  int n = 0;  // entries, without the padding
 };
 template <typename F>
 int grow_tile(const bc_plan* P, int q, int q1, int L, int plane, F entries, TileBox& T,
@@ -1327,18 +1344,21 @@ int grow_tile(const bc_plan* P, int q, int q1, int L, int plane, F entries, Tile
       E.box[at] = ents[t].sel * A + (ents[t].i - T.imin) + (ents[t].j - T.jmin) * bw;
       E.w[at] = ents[t].w;
     }
-  return (double)ents.size() < kMinTileReuse * A * T.nsel ? -nq : nq;
+  E.n = (int)ents.size();
+  return nq;
 }
 
-// Staged CSR rows of component ci of sub-matrix s.  Returns false (the
-// component keeps the per-lane path) when some row does not qualify.
-bool emit_csr_tiles(bc_plan* P, const Sub& s, int ci, const Item& proto, std::vector<Item>& out) {
+// Staged CSR rows of component ci of sub-matrix s; adds to `sums`.  Returns
+// false (the component keeps the per-lane path) when some row does not qualify.
+bool emit_csr_tiles(bc_plan* P, const Sub& s, int ci, const Item& proto, std::vector<Item>& out,
+                    TileSums& sums) {
   const int L = P->blocks[s.block].nlevels;
   const int w = s.ell_w;
   // rows of one entry read nothing twice: they take the shorter chain
   const auto nnz0 = P->csr_nnz.begin() + (s.table + ci * s.vol);
   if (*std::max_element(nnz0, nnz0 + s.vol) <= 1) return false;
   std::vector<Item> tiles;
+  TileSums mine;
   TileEntries all, E;
   auto entries = [&](int q, auto f) {
     const size_t e0 = (size_t)s.ell_base + ((size_t)ci * s.vol + q) * w;
@@ -1348,7 +1368,7 @@ bool emit_csr_tiles(bc_plan* P, const Sub& s, int ci, const Item& proto, std::ve
   for (int q0 = 0; q0 < s.vol;) {
     TileBox T;
     const int nq = grow_tile(P, q0, s.vol, L, kPlaneCsr, entries, T, E);
-    if (nq <= 0) return false;
+    if (nq == 0) return false;
     Item it = proto;
     it.src_org = (int32_t)(P->tile_box.size() + all.box.size());
     // rows of blocks of 8 entries read whole blocks: pad the last one
@@ -1360,8 +1380,10 @@ bool emit_csr_tiles(bc_plan* P, const Sub& s, int ci, const Item& proto, std::ve
     all.box.insert(all.box.end(), E.box.begin(), E.box.end());
     all.w.insert(all.w.end(), E.w.begin(), E.w.end());
     q0 += nq;
+    mine += {1, nq, E.n, T.cells() * T.nsel};
   }
   if (P->tile_box.size() + all.box.size() > INT32_MAX) return false;
+  sums += mine;
   P->tile_box.insert(P->tile_box.end(), all.box.begin(), all.box.end());
   P->tile_w.insert(P->tile_w.end(), all.w.begin(), all.w.end());
   out.insert(out.end(), tiles.begin(), tiles.end());
@@ -1396,8 +1418,8 @@ bool emit_adj_tiles(bc_plan* P, int r0, int nrows, const Item& proto, int chunk,
   for (int q0 = 0; q0 < nrows;) {
     TileBox T;
     const int nq = grow_tile(P, q0, nrows, L, kPlaneAdj, entries, T, E);
-    if (nq <= 0) {
-      q0 += std::max(1, -nq);
+    if (nq == 0 || E.n < kMinTileReuse * (double)(T.cells() * T.nsel)) {
+      q0 += std::max(1, nq);
       continue;
     }
     flush(q0);
@@ -1486,9 +1508,10 @@ void build_items(bc_plan* P) {
   // rows with levels far apart in memory, staged below if that pays
   struct Rows {
     size_t sub;
+    int ci;
     Item proto;
   };
-  std::vector<Rows> interp_rows;
+  std::vector<Rows> interp_rows, csr_rows;
   for (size_t si = 0; si < P->subs.size(); ++si) {
     const Sub& s = P->subs[si];
     const bc_block& B = P->blocks[s.block];
@@ -1531,7 +1554,7 @@ void build_items(bc_plan* P) {
           if (mode < 2 || P->opts.unstaged_rows)
             table_emit(out, it, B, s.vol);
           else
-            interp_rows.push_back({si, it});
+            interp_rows.push_back({si, (int)ci, it});
           break;
         }
         case BC_CSR: {
@@ -1544,11 +1567,11 @@ void build_items(bc_plan* P) {
             const bc_block& S = P->blocks[P->slot_block[it.src_slot]];
             it.src_ls = (int32_t)(S.nlevels > 1 ? S.level_stride : 0);
           }
-          // levels far apart in memory: stage each tile's column box
           const int mode = table_mode(B, P->opts.unit_order, level_chunk(P, it.kind));
-          if (mode < 2 || P->opts.unstaged_rows ||
-              !emit_csr_tiles(P, s, (int)ci, it, out))
+          if (mode < 2 || P->opts.unstaged_rows)
             table_emit(out, it, B, s.vol);
+          else
+            csr_rows.push_back({si, (int)ci, it});
           break;
         }
       }
@@ -1573,12 +1596,21 @@ void build_items(bc_plan* P) {
       else
         per_lane(rows[k]);
     }
+    return staged;
   };
   stage_rows(interp_rows,
              [&](const Rows& r, std::vector<Item>& out, TileSums& sums) {
                return emit_tiles(P, P->subs[r.sub], r.proto, out, sums);
              },
              keep_interp_tiles);
+  if (!stage_rows(csr_rows,
+                  [&](const Rows& r, std::vector<Item>& out, TileSums& sums) {
+                    return emit_csr_tiles(P, P->subs[r.sub], r.ci, r.proto, out, sums);
+                  },
+                  keep_csr_tiles)) {
+    P->tile_box.clear();
+    P->tile_w.clear();
+  }
   // order: by kind, then sub-matrix (per-sub and per-kind ranges contiguous)
   P->items.clear();
   P->sub_begin.assign(P->subs.size(), 0);
