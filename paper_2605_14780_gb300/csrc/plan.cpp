@@ -1391,9 +1391,18 @@ bool emit_csr_tiles(bc_plan* P, const Sub& s, int ci, const Item& proto, std::ve
 }
 
 // Staged transpose rows [r0, r0 + nrows) (one data slot; per-lane rows in
-// chunks of `chunk` levels).  Rows that cannot be staged keep the per-lane
-// gather (items of up to 32 rows and one level chunk).  Returns false,
-// emitting nothing, when no row can.
+// chunks of `chunk` levels).  Rows that cannot be staged, and those of tiles
+// with less than kAdjTileUnits (row, level group) units for the 32 lanes, keep
+// the per-lane gather (items of up to 32 rows and one level chunk).  Returns
+// false, emitting nothing, when no row can be staged.
+//
+// Short tiles leave lanes idle, the more so in FP64 with its one group of
+// levels: 6 x 384^2 x 32 levels, rows that 16-entry ghosts in groups of eight
+// read, FP64 95 us with every such tile staged at the earlier tile size, 123 at
+// the present one, 36 so (16 units: 38); groups of 16 74, 69, 36 (60); random
+// 4-point nodes, three components, 213, 364, 143.  Full tiles are not touched
+// (6 x 600^2 panel edges 108 us, per lane 119).
+constexpr int kAdjTileUnits = 24;
 bool emit_adj_tiles(bc_plan* P, int r0, int nrows, const Item& proto, int chunk, int L,
                     std::vector<Item>& out) {
   std::vector<Item> items;
@@ -1404,6 +1413,7 @@ bool emit_adj_tiles(bc_plan* P, int r0, int nrows, const Item& proto, int chunk,
       f(P->aent_slot[(size_t)e], P->aent_off[(size_t)e], P->aent_w[(size_t)e]);
   };
   bool staged = false;
+  const int groups = (tile_levels(P, L, false) + kTileLevels - 1) / kTileLevels;
   int plain0 = 0;  // first row of the pending unstaged ones
   auto flush = [&](int end) {
     for (int q0 = plain0; q0 < end; q0 += kTileCells)
@@ -1418,7 +1428,7 @@ bool emit_adj_tiles(bc_plan* P, int r0, int nrows, const Item& proto, int chunk,
   for (int q0 = 0; q0 < nrows;) {
     TileBox T;
     const int nq = grow_tile(P, q0, nrows, L, kPlaneAdj, entries, T, E);
-    if (nq == 0 || E.n < kMinTileReuse * (double)(T.cells() * T.nsel)) {
+    if (nq * groups < kAdjTileUnits || E.n < kMinTileReuse * (double)(T.cells() * T.nsel)) {
       q0 += std::max(1, nq);
       continue;
     }

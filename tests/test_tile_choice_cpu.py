@@ -90,3 +90,11 @@ def test_a_short_last_tile_keeps_the_others_staged(n):
     tiles = 3 * -(-n // 32)
     assert _plan(w)["nitems"] <= tiles * 2  # 8 levels, four a stage
     assert _staged(w)
+
+
+@pytest.mark.parametrize("dtype,group,staged", [
+    ("f32", 4, False), ("f32", 8, False), ("f32", 16, True), ("f32", 32, True),
+    ("f64", 4, False), ("f64", 8, False), ("f64", 32, True)])
+def test_transpose_rows(dtype, group, staged):
+    # a group of g ghosts reads a column of g + 3 cells: as many rows
+    assert _staged(grouped_interp(group, dtype), "nitems_adjoint") == staged
