@@ -2382,19 +2382,28 @@ bc_status build_fusion(bc_plan* P) {
     cta += f.tiles + ((F - D) * B.nlevels + kFuseThreads - 1) / kFuseThreads;
   }
   P->fuse_ctas = cta;
-  // Box path: planes per tile.  A tile's cost is its planes plus the two it
-  // only sums (and about eight planes' worth of start-up), the grid's the
-  // tiles of the fullest SM: 16 blocks of 128^3 take 32 planes (2048 tiles).
+  // Box path: planes per tile, an even number (the outputs come in pairs of
+  // planes, so their rounding does not depend on it).  A tile costs its planes
+  // plus the two it only sums, as FP64 issue where an SM holds several (1.05 us
+  // a plane) and as a chain of latencies where it holds one (5.4 us and 4 us a
+  // plane; of a wave after the first, eight tiles an SM, 0.7 shows).  One block
+  // of 128^3: 142 us with 32 planes, which leave SMs without a tile, 47 with the
+  // 4 taken here (general kernel 114); 16 blocks: 492 with the 16 taken, 505
+  // with 32, 557 with 4; one block of 16^3: 18 with 2, 26 with 4.  Over 38 grids
+  // measured the choice is the best one or within 2 % of it but for one (12 %).
   {
     double best = 0;
-    int bz = 4;
-    for (int z : {4, 6, 8, 12, 16, 24, 32, 48, 64}) {
+    int bz = 2;
+    for (int z : {2, 4, 6, 8, 12, 16, 24, 32, 48, 64}) {
       int64_t tiles = 0;
       for (const FuseSlot& f : slots)
         tiles += (int64_t)((f.n[0] + kBoxX - 1) / kBoxX) * ((f.n[1] + kBoxY - 1) / kBoxY) *
                  ((f.n[2] + z - 1) / z) * f.L;
-      const double cost = (double)((tiles + P->num_sms - 1) / P->num_sms) * (z + 1.2 + 8.0);
-      if (z == 4 || cost < best) {
+      const int sms = std::max(1, P->num_sms);
+      const double issue = (double)((tiles + sms - 1) / sms) * (z + 1.2) * 1.05;
+      const double waves = 1 + 0.7 * (double)((tiles + 8 * sms - 1) / (8 * sms) - 1);
+      const double cost = std::hypot(issue, (5.4 + 4.05 * z) * waves);
+      if (z == 2 || cost < best) {
         best = cost;
         bz = z;
       }
