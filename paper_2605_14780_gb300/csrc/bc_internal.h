@@ -272,15 +272,14 @@ struct FuseStencil {
 };
 cudaError_t launch_fused(int dtype, const FuseCtx& F, const FuseStencil& st, void* const* slots,
                          void* const* outs, int64_t nctas, cudaStream_t s);
-// Box path: CTAs of kBoxThreads, one per tile of kBoxX x kBoxY cells and
+// Box path (FP64): CTAs of kBoxThreads, one per tile of kBoxX x kBoxY cells and
 // FuseSlot::bz planes and level; reads the ghosts from memory (filled by an
 // earlier launch on the stream).
 constexpr int kBoxThreads = 64;
 constexpr int kBoxTy = 4;  // outputs of a thread along y (2 along x)
 constexpr int kBoxX = 32, kBoxY = kBoxThreads / 16 * kBoxTy;
-cudaError_t launch_fused_box(int dtype, const FuseCtx& F, const FuseStencil& st,
-                             void* const* slots, void* const* outs, int64_t nctas,
-                             cudaStream_t s);
+cudaError_t launch_fused_box(const FuseCtx& F, const FuseStencil& st, void* const* slots,
+                             void* const* outs, int64_t nctas, cudaStream_t s);
 
 // Box packing (pack.cu): one descriptor per box; CTAs take tiles of at most
 // nc cells x nl levels of one component, {box, component, first cell, first

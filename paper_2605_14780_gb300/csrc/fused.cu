@@ -249,39 +249,33 @@ __global__ void __launch_bounds__(kFuseThreads)
 // pairs; a ring of four planes with their halo sits in shared memory (20 KB
 // in FP64, eight CTAs an SM: while one waits for its planes the others keep
 // the pipe busy; 4 warps a CTA: 2 % longer, 1 warp: 1 %).  The sums associate
-// differently from the general kernel's (against sums in higher precision
-// they are the closer ones: 1.4e-16 to 2.2e-16 of the result's norm for the
-// operator below); a value that is not finite is summed again in the general
-// order from the ring, so infinities, NaNs and overflow come out as there.
+// differently from the general kernel's: against sums in higher precision they
+// are the closer ones for random values (1.4e-16 to 2.2e-16 of the result's norm
+// for the operator below), for smooth fields on a large mean 0.9 to 1.4 times as
+// far off.  A value that is not finite is summed again in the general order from
+// the ring, so infinities, NaNs and overflow come out as there.
 //
-// 27-point operator (26, -1) on 16 blocks of 128^3 FP64, fill included:
-// 1579 -> 474 us, the FP64 pipe 75 % busy.
-template <typename T>
-__device__ __forceinline__ void cp_async_cell(T* smem, const T* gmem) {
+// 27-point operator (26, -1), FP64, fill included: 16 blocks of 128^3 1576 -> 492
+// us (6.25 instructions a value take 0.69 of the pipe's rate), one 114 -> 47,
+// four of 64^3 63 -> 34, one of 16^3 even at 18 (build_fusion chooses the planes
+// per tile).
+__device__ __forceinline__ void cp_async_cell(double* smem, const double* gmem) {
   const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
-  if constexpr (sizeof(T) == 4)
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(sa), "l"(gmem) : "memory");
-  else
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(sa), "l"(gmem) : "memory");
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(sa), "l"(gmem) : "memory");
 }
 
 constexpr int kBoxPitch = kBoxX + 2, kBoxPlane = kBoxPitch * (kBoxY + 2);
 constexpr int kBoxCtas = 512 / kBoxThreads;  // 16 warps an SM
 
-template <typename T> struct Pair2;
-template <> struct Pair2<double> { using type = double2; };
-
 // 3 x 3 sums of one staged plane for a thread's 2 x 4 cells; `c`: the
 // staged value one row above and one cell before the thread's first
-template <typename T>
-__device__ __forceinline__ void plane_sums(const T* c, T (&P)[2 * kBoxTy]) {
-  using V = typename Pair2<T>::type;
-  T r[kBoxTy + 2][2];
+__device__ __forceinline__ void plane_sums(const double* c, double (&P)[2 * kBoxTy]) {
+  double r[kBoxTy + 2][2];
 #pragma unroll
   for (int j = 0; j < kBoxTy + 2; ++j) {
-    const V a = *reinterpret_cast<const V*>(c + j * kBoxPitch);
-    const V b = *reinterpret_cast<const V*>(c + j * kBoxPitch + 2);
-    const T s = a.y + b.x;
+    const double2 a = *reinterpret_cast<const double2*>(c + j * kBoxPitch);
+    const double2 b = *reinterpret_cast<const double2*>(c + j * kBoxPitch + 2);
+    const double s = a.y + b.x;
     r[j][0] = a.x + s;
     r[j][1] = s + b.y;
   }
@@ -289,7 +283,7 @@ __device__ __forceinline__ void plane_sums(const T* c, T (&P)[2 * kBoxTy]) {
   for (int x = 0; x < 2; ++x)
 #pragma unroll
     for (int j = 0; j < kBoxTy; j += 2) {
-      const T s = r[j + 1][x] + r[j + 2][x];
+      const double s = r[j + 1][x] + r[j + 2][x];
       P[2 * j + x] = r[j][x] + s;
       P[2 * (j + 1) + x] = s + r[j + 3][x];
     }
@@ -306,12 +300,12 @@ __device__ __forceinline__ double flip_sign(double v, unsigned flip) {
 }
 
 // UNIT: |a| = 1, a x S is S or -S
-template <typename T, bool UNIT>
+template <bool UNIT>
 __global__ void __launch_bounds__(kBoxThreads, kBoxCtas)
     k_fused_box(FuseCtx F, FuseStencil st, void* const* slots, void* const* outs) {
   __shared__ FuseSlot S;
   __shared__ int si;
-  __shared__ __align__(16) T ring[4][kBoxPlane];
+  __shared__ __align__(16) double ring[4][kBoxPlane];
   const int tid = threadIdx.x;
   if (tid == 0) {
     int lo = 0, hi = F.nslots - 1;  // the last slot whose first CTA is <= blockIdx.x
@@ -336,7 +330,7 @@ __global__ void __launch_bounds__(kBoxThreads, kBoxCtas)
   const int warp = tid >> 5, lane = tid & 31;
   const int64_t s0 = S.s[0], s1 = S.s[1], s2 = S.s[2];
   const int64_t org = cell_off(S, i0, j0, k0) + (int64_t)l * S.ls;
-  const T* x = static_cast<const T*>(slots[si]) + org;
+  const double* x = static_cast<const double*>(slots[si]) + org;
 
   // planes k and k + 1 with their halo into the ring (plane k in slot k & 3),
   // a warp a row; cells past the full region only border outputs past the
@@ -345,17 +339,17 @@ __global__ void __launch_bounds__(kBoxThreads, kBoxCtas)
   auto stage = [&](int k) {
     for (int r = warp; r < 2 * (kBoxY + 2); r += kBoxThreads / 32) {
       const int z = r >= kBoxY + 2, j = r - z * (kBoxY + 2) - 1, kk = k + z;
-      T* dst = ring[kk & 3] + (j + 1) * kBoxPitch;
+      double* dst = ring[kk & 3] + (j + 1) * kBoxPitch;
       const bool row = j < jend && kk < S.n[2] + S.h[2];
-      const T* src = x + ((int64_t)(kk - k0) * s2 + (int64_t)j * s1);
+      const double* src = x + ((int64_t)(kk - k0) * s2 + (int64_t)j * s1);
 #pragma unroll
       for (int u = 0; u < 2; ++u) {
         const int li = lane + 32 * u;
         if (li >= kBoxPitch) break;
         if (row && li - 1 < iend)
-          cp_async_cell<T>(dst + li, src + (int64_t)(li - 1) * s0);
+          cp_async_cell(dst + li, src + (int64_t)(li - 1) * s0);
         else
-          dst[li] = T(0);
+          dst[li] = 0.0;
       }
     }
     asm volatile("cp.async.wait_all;\n" ::: "memory");
@@ -367,45 +361,45 @@ __global__ void __launch_bounds__(kBoxThreads, kBoxCtas)
   // a warp whose rows all lie past the block has nothing to sum
   const bool work = j0 + warp * 2 * kBoxTy < S.n[1];
   const int nx = S.n[0] - i0 - cx, ny = S.n[1] - j0 - cy;  // this thread's cells in the block
-  T* out = static_cast<T*>(outs[si]) + (org + cx * s0 + cy * s1);
-  const T a = (T)st.a, d = (T)st.d;
+  double* out = static_cast<double*>(outs[si]) + (org + cx * s0 + cy * s1);
+  const double a = st.a, d = st.d;
   const unsigned flip = st.a < 0 ? 0x80000000u : 0u;
 
   // the outputs of plane k from the box sums b
-  auto put = [&](int k, const T (&b)[2 * kBoxTy]) {
-    const T* c = ring[k & 3] + at + kBoxPitch + 1;
-    T* o = out + (int64_t)(k - k0) * s2;
+  auto put = [&](int k, const double (&b)[2 * kBoxTy]) {
+    const double* c = ring[k & 3] + at + kBoxPitch + 1;
+    double* o = out + (int64_t)(k - k0) * s2;
 #pragma unroll
     for (int j = 0; j < kBoxTy; ++j)
 #pragma unroll
       for (int xx = 0; xx < 2; ++xx) {
-        const T x0 = c[j * kBoxPitch + xx], s = b[2 * j + xx];
-        T v = UNIT ? fma(d, x0, flip_sign(s, flip)) : fma(a, s, d * x0);
+        const double x0 = c[j * kBoxPitch + xx], s = b[2 * j + xx];
+        double v = UNIT ? fma(d, x0, flip_sign(s, flip)) : fma(a, s, d * x0);
         if (!finite_value(v)) {
-          v = T(0);
+          v = 0.0;
           for (int p = 0; p < st.n; ++p)
-            v = fma((T)st.c[p],
+            v = fma(st.c[p],
                     ring[(k + st.o[p][2]) & 3]
-                    [at + (j + 1 + st.o[p][1]) * kBoxPitch + xx + 1 + st.o[p][0]],
+                        [at + (j + 1 + st.o[p][1]) * kBoxPitch + xx + 1 + st.o[p][0]],
                     v);
         }
         if (xx < nx && j < ny) o[j * s1 + xx * s0] = v;
       }
   };
 
-  T p0[2 * kBoxTy], p1[2 * kBoxTy];  // plane sums of k - 1 and k
+  double p0[2 * kBoxTy], p1[2 * kBoxTy];  // plane sums of k - 1 and k
   stage(k0 - 1);
   __syncthreads();
   if (work) {
-    plane_sums<T>(ring[(k0 - 1) & 3] + at, p0);
-    plane_sums<T>(ring[k0 & 3] + at, p1);
+    plane_sums(ring[(k0 - 1) & 3] + at, p0);
+    plane_sums(ring[k0 & 3] + at, p1);
   }
   for (int k = k0; k < k1; k += 2) {
     stage(k + 1);
     __syncthreads();
     if (work) {
-      T p2[2 * kBoxTy], b[2 * kBoxTy];
-      plane_sums<T>(ring[(k + 1) & 3] + at, p2);
+      double p2[2 * kBoxTy], b[2 * kBoxTy];
+      plane_sums(ring[(k + 1) & 3] + at, p2);
 #pragma unroll
       for (int q = 0; q < 2 * kBoxTy; ++q) {
         p1[q] += p2[q];         // planes k and k + 1, shared by both outputs
@@ -414,7 +408,7 @@ __global__ void __launch_bounds__(kBoxThreads, kBoxCtas)
       }
       put(k, b);
       if (k + 1 < k1) {
-        plane_sums<T>(ring[(k + 2) & 3] + at, p2);
+        plane_sums(ring[(k + 2) & 3] + at, p2);
 #pragma unroll
         for (int q = 0; q < 2 * kBoxTy; ++q) {
           b[q] = p1[q] + p2[q];
@@ -439,13 +433,11 @@ cudaError_t launch_fused(int dtype, const FuseCtx& F, const FuseStencil& st, voi
   return cudaGetLastError();
 }
 
-cudaError_t launch_fused_box(int dtype, const FuseCtx& F, const FuseStencil& st,
-                             void* const* slots, void* const* outs, int64_t nctas,
-                             cudaStream_t s) {
+cudaError_t launch_fused_box(const FuseCtx& F, const FuseStencil& st, void* const* slots,
+                             void* const* outs, int64_t nctas, cudaStream_t s) {
   if (nctas <= 0) return cudaSuccess;
   const bool unit = st.a == 1.0 || st.a == -1.0;
-  if (dtype != 1) return cudaErrorInvalidValue;  // FP64 plans only
-  auto* kernel = unit ? k_fused_box<double, true> : k_fused_box<double, false>;
+  auto* kernel = unit ? k_fused_box<true> : k_fused_box<false>;
   kernel<<<(unsigned)nctas, kBoxThreads, 0, s>>>(F, st, slots, outs);
   return cudaGetLastError();
 }

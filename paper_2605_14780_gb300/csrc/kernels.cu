@@ -1590,7 +1590,7 @@ __global__ void __launch_bounds__(THREADS, (Occ<FAM, THREADS>::kMinBlocks))
   if (Stage<FAM, THREADS>::kWarps) P.stage = warp * c.stage_warp;
   __syncwarp();
   // the adjoint's zero pass starts while the gather's last CTAs run
-  // (launch_after): it reads its items by then, and stores after the gather
+  // (kGridAfter): it reads its items by then, and stores after the gather
   if constexpr (FAM == FAM_STRUCT) asm volatile("griddepcontrol.wait;\n" ::: "memory");
   if constexpr (FAM == FAM_ADJ) asm volatile("griddepcontrol.launch_dependents;\n");
   run_work<T, FAM>(sit[warp], P, c, lane);

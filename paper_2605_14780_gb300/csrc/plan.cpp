@@ -3522,8 +3522,7 @@ bc_status bc_apply_stencil(bc_plan* plan, void* const* slot_ptrs, void* const* o
       e = launch_family(plan->dtype, f, c, plan->d_fam[f], (int)plan->fam_items[f].size(),
                         plan->opts.threads, 0, plan->staged[f], s);
     if (e == cudaSuccess)
-      e = launch_fused_box(plan->dtype, plan->fuse_ctx, st, slot_ptrs, out_ptrs,
-                           plan->fuse_box_ctas, s);
+      e = launch_fused_box(plan->fuse_ctx, st, slot_ptrs, out_ptrs, plan->fuse_box_ctas, s);
   } else {
     e = launch_fused(plan->dtype, plan->fuse_ctx, st, slot_ptrs, out_ptrs, plan->fuse_ctas, s);
   }
