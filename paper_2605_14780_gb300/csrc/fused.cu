@@ -256,7 +256,7 @@ __global__ void __launch_bounds__(kFuseThreads)
 // the ring, so infinities, NaNs and overflow come out as there.
 //
 // 27-point operator (26, -1), FP64, fill included: 16 blocks of 128^3 1576 -> 492
-// us (6.25 instructions a value take 0.69 of the pipe's rate), one 114 -> 47,
+// us (6.25 instructions a value take 0.68 of the pipe's rate), one 114 -> 47,
 // four of 64^3 63 -> 34, one of 16^3 even at 18 (build_fusion chooses the planes
 // per tile).
 __device__ __forceinline__ void cp_async_cell(double* smem, const double* gmem) {
